@@ -6,9 +6,9 @@
 // one 128-bit load, the one-column halo comes from the neighbouring lane by
 // shuffle, rows slide through registers so each input row is loaded once per
 // strip, the next rows are loaded before the current one is used, and
-// outputs leave as 128-bit (or 64-bit) streaming stores.  Shapes the vector
-// path does not cover use a thread-per-output scalar path with the same
-// arithmetic.
+// outputs leave as 128-bit (or 64-bit) streaming stores.  Rows that are not
+// 16-byte multiples, and unaligned tensors, take the flat path (FlatRows
+// below) with the same arithmetic.
 #pragma once
 #include "hf_device.cuh"
 
@@ -32,6 +32,103 @@ struct ItemCursor {
 };
 
 // ------------------------------------------------------------------------
+// The flat path, for rows of any length.  The rows of all planes are one
+// sequence; a work item is R consecutive rows, whatever planes they belong
+// to, and its pixels i = 0 .. R*W-1 go to lanes in memory order, so a row of
+// 7 or 75 values leaves no lane idle and neighbours are at constant offsets
+// (-W-1 .. W+1) from a pixel.  An item's input rows with their halo are one
+// contiguous range: with a ring they arrive as one bulk copy, its ends
+// rounded out to 16 bytes (the tensor's last values, past its last multiple
+// of four, are patched in with plain loads); without one the lanes load them
+// from global memory.  Only the division of a pixel's index by the row
+// length remains, a multiply and a shift (indices stay below 1024).
+//
+// The bound is HBM; one 32-pixel step of upsample moves 640 bytes in about
+// 45 issue slots, where an SM has about 108 for them.  It replaces paths of
+// one thread per output with two 64-bit divisions each.  On one GB300, before
+// -> with it: upsample 8x64x75x75 + max pool 8x64x147x147 fused 287 -> 27.7
+// us, im2col 8x64x112x112 alone 309 -> 46.2 us (5.6 TB/s), batch-norm
+// 64x512x7x7 + im2col 32x256x14x14 fused 243 -> 22.3 us.
+struct FlatRows {
+    unsigned W, H, R;    // values per row, rows per plane, rows per item
+    unsigned rows;       // rows of all planes
+    unsigned mw, mh;     // ceil(2^20 / W), ceil(2^21 / H)
+    static constexpr unsigned kMaxValues = 1014;   // values of an item (i * (W - 1) < 2^20)
+
+    // rmax: rows an item may have; warps: of the grid; R is a multiple of
+    // `multiple`.  Items are as large as rmax and as even as the number of
+    // warps allows.
+    __device__ void init(unsigned w, unsigned h, unsigned rows_, unsigned rmax, unsigned warps, unsigned multiple)
+    {
+        W = w;
+        H = h;
+        rows = rows_;
+        const unsigned each = (rows + warps - 1) / warps;      // rows per warp
+        const unsigned turns = (each + rmax - 1) / rmax;       // items per warp
+        R = (each + turns - 1) / turns;
+        R = min((R + multiple - 1) / multiple * multiple, rmax);
+        mw = ((1u << 20) + W - 1) / W;
+        mh = ((1u << 21) + H - 1) / H;
+    }
+    __device__ unsigned items() const { return (rows + R - 1) / R; }
+    // row of pixel i of an item; plane (counted from the item's first) of
+    // row t of that plane's run of rows, t < H + R
+    __device__ unsigned row_of(unsigned i) const { return R == 1 ? 0u : (i * mw) >> 20; }
+    __device__ unsigned plane_of(unsigned t) const { return H <= 1024 ? (t * mh) >> 21 : (t >= H ? 1u : 0u); }
+};
+
+// Reads of an item's values at offsets from its first pixel: from the stage,
+// where every offset within the halo is inside the stage (values outside
+// the tensor are never used), or from global memory where `ok`.
+struct FlatStage {
+    const float *p;
+    __device__ float operator()(int off, bool) const { return p[off]; }
+};
+struct FlatGlobal {
+    const float *p;
+    __device__ float operator()(int off, bool ok) const { return ok ? __ldg(p + off) : 0.f; }
+};
+
+// The stage layout of values [lo, hi) of x (lo may be negative, hi past the
+// end): stage float k holds value base + k, base = lo rounded down to a
+// multiple of four.  Lane 0 copies what lies in [0, total / 4 * 4).
+struct FlatCopy {
+    int64_t base, src, end;   // first value of the stage, values copied [src, end)
+    __device__ FlatCopy(int64_t lo, int64_t hi, int64_t total)
+    {
+        base = lo & ~(int64_t)3;
+        src = base > 0 ? base : 0;
+        const int64_t up = (hi + 3) & ~(int64_t)3, most = total & ~(int64_t)3;
+        end = up < most ? up : most;
+    }
+    __device__ void fill(const WarpRing &r, int st, const float *x) const
+    {
+        const unsigned bytes = end > src ? (unsigned)(end - src) * 4u : 0u;
+        r.expect(st, bytes);
+        if (bytes) r.copy(st, (unsigned)(src - base) * 4u, x + src, bytes);
+    }
+    // all lanes, once the stage has landed: the tensor's last values
+    __device__ void patch(unsigned char *stage, const float *x, int64_t hi, int64_t total, int lane) const
+    {
+        const int64_t last = total & ~(int64_t)3;
+        const int64_t upto = hi < total ? hi : total;
+        if (upto > last) {
+            const int64_t first = last > base ? last : base;
+            if (first + lane < upto) reinterpret_cast<float *>(stage)[first + lane - base] = __ldg(x + first + lane);
+            __syncwarp();
+        }
+    }
+};
+// The range of the flat path's 32-bit rows, offsets and warp counts.
+__device__ __forceinline__ bool flat_range(int64_t rows, int64_t W, const Ctx &cx)
+{
+    return rows < ((int64_t)1 << 31) && W < ((int64_t)1 << 29) && (int64_t)cx.grid * (cx.nthreads >> 5) < ((int64_t)1 << 31);
+}
+// Floats of a stage that an item's halo and the rounding take: base is up to
+// three below lo, the copy's end up to three past hi.
+constexpr unsigned kFlatPad = 8;
+
+// ------------------------------------------------------------------------
 // Bilinear x2, half-pixel centres.  Along one axis of length L, output 2i
 // blends input i-1 and i with weights 1/4, 3/4 (output 0 is input 0) and
 // output 2i+1 blends i and i+1 with 3/4, 1/4 (output 2L-1 is input L-1).
@@ -49,11 +146,29 @@ struct BodyUpsample {
     static constexpr bool kRingItem = true;
     static constexpr unsigned kRingMinBytes = 4096;   // the stage: one item
 
-    // strips of whole rows (W <= 128, 16-byte rows) arrive as one bulk copy
+    // Which path: 16-byte rows of 64 values or more go to strips of whole
+    // rows (four columns a lane), the others to the flat path.  Strips leave
+    // lanes idle below 128 columns: 2^23 values in images of W = 8 / 16 /
+    // 32 / 40 / 56 / 64 columns took 181 / 83 / 49 / 41 / 35 / 33 us alone,
+    // the flat path 37 / 35 / 34 / 36 / 35 / 35.
+    // Rows of 129 to 252 columns are too long for a strip's stage, but two
+    // rows with their halo still fit a flat item's: 57 us on registers, 51
+    // flat (W = 224, four warps an SM; 39 and 37 us at full occupancy).
+    // Longer ones keep the register path (W = 400: 39 us, 47 flat).
+    static constexpr int kStripCols = 64;
+    static __host__ __device__ bool rows16(const Args &a)
+    {
+        return (a.W & 3) == 0 && aligned16(a.x) && aligned16(a.y);
+    }
+    static __host__ __device__ bool strips(const Args &a)
+    {
+        return rows16(a) && a.W >= kStripCols && (a.W <= 128 || 4u * a.W + kFlatPad > kRingMinBytes / 4);
+    }
+    // a strip's rows (W <= 128) or a flat item's arrive as one bulk copy
     static __host__ bool uses_ring(const Args &a)
     {
-        return (int64_t)a.P * a.H * a.W > 0 && (a.W & 3) == 0 && a.W <= 128 && aligned16(a.x) &&
-               aligned16(a.y);
+        if ((int64_t)a.P * a.H * a.W <= 0) return false;
+        return strips(a) ? a.W <= 128 : aligned16(a.x) && 3u * a.W + kFlatPad <= kRingMinBytes / 4;
     }
 
     static __host__ size_t workspace_bytes(const Args &) { return 0; }
@@ -247,6 +362,89 @@ struct BodyUpsample {
         return true;
     }
 
+    // One item of the flat path: pixel i gives the outputs (2r, 2r+1) x
+    // (2c, 2c+1); in memory they start at 4*i - 2*c from the item's first.
+    template <class Get>
+    static __device__ __forceinline__ void flat_item(const Args &a, const FlatRows &f, unsigned g0, unsigned n,
+                                                     const Get &get)
+    {
+        const int W = (int)f.W;
+        const unsigned r0 = g0 % f.H;
+        float *y0 = a.y + 4 * (int64_t)g0 * W;
+        const bool y8 = (reinterpret_cast<uintptr_t>(a.y) & 7u) == 0;
+#pragma unroll 2
+        for (unsigned i = lane_id(); i < n; i += 32) {
+            const unsigned lr = f.row_of(i), c = i - lr * f.W, t = r0 + lr;
+            const unsigned r = t - f.plane_of(t) * f.H;
+            const bool le = c == 0, re = c == f.W - 1, te = r == 0, be = r == f.H - 1;
+            auto hrow = [&](int off, bool ok, float &h0, float &h1) {
+                const float C = get(off, ok), L = get(off - 1, ok && !le), R = get(off + 1, ok && !re);
+                h0 = le ? C : blend(C, L);
+                h1 = re ? C : blend(C, R);
+            };
+            float u0, u1, c0, c1, d0, d1;
+            hrow((int)i - W, !te, u0, u1);
+            hrow((int)i, true, c0, c1);
+            hrow((int)i + W, !be, d0, d1);
+            const float2 e = make_float2(te ? c0 : blend(c0, u0), te ? c1 : blend(c1, u1));
+            const float2 o = make_float2(be ? c0 : blend(c0, d0), be ? c1 : blend(c1, d1));
+            float *ye = y0 + (4 * (int64_t)i - 2 * c), *yo = ye + 2 * W;
+            if (y8) {
+                stcs2(ye, e);
+                stcs2(yo, o);
+            } else {
+                __stcs(ye, e.x);
+                __stcs(ye + 1, e.y);
+                __stcs(yo, o.x);
+                __stcs(yo + 1, o.y);
+            }
+        }
+    }
+
+    static __device__ bool flat_ring(const Args &a, const Ctx &cx)
+    {
+        const int64_t rows = (int64_t)a.P * a.H, total = rows * a.W;
+        const int nw = cx.nthreads >> 5;
+        const int64_t gw = (int64_t)cx.block * nw + (cx.tid >> 5), GW = (int64_t)cx.grid * nw;
+        const unsigned W = (unsigned)a.W, slots = min(cx.ring_stage, 4096u) / 4;
+        if (!aligned16(a.x) || 3 * W + kFlatPad > slots || !WarpRing::available(cx, 0)) return false;
+        FlatRows f;
+        f.init(W, a.H, (unsigned)rows, min((slots - kFlatPad) / W - 2, FlatRows::kMaxValues / W), (unsigned)GW, 1);
+        WarpRing r;
+        r.init(cx, 0);
+        auto copy = [&](int64_t it) {
+            const int64_t g0 = it * f.R;
+            return FlatCopy((g0 - 1) * W - 1, (min(g0 + (int64_t)f.R, rows) + 1) * W + 1, total);
+        };
+        ring_stream(
+            r, gw, GW, f.items(), [&](int st, int64_t it) { copy(it).fill(r, st, a.x); },
+            [&](unsigned char *stage, int64_t it) {
+                const int64_t g0 = it * f.R, g1 = min(g0 + (int64_t)f.R, rows);
+                const FlatCopy k = copy(it);
+                k.patch(stage, a.x, (g1 + 1) * W + 1, total, r.lane);
+                flat_item(a, f, (unsigned)g0, (unsigned)(g1 - g0) * W,
+                          FlatStage{reinterpret_cast<const float *>(stage) + (g0 * W - k.base)});
+            });
+        r.finish();
+        return true;
+    }
+
+    // The same items without a ring.
+    static __device__ void flat_global(const Args &a, const Ctx &cx)
+    {
+        const int64_t rows = (int64_t)a.P * a.H;
+        const int nw = cx.nthreads >> 5;
+        const int64_t gw = (int64_t)cx.block * nw + (cx.tid >> 5), GW = (int64_t)cx.grid * nw;
+        const unsigned W = (unsigned)a.W;
+        FlatRows f;
+        f.init(W, a.H, (unsigned)rows, max(1u, FlatRows::kMaxValues / W), (unsigned)GW, 1);
+        for (int64_t it = gw; it < f.items(); it += GW) {
+            const int64_t g0 = it * f.R, g1 = min(g0 + (int64_t)f.R, rows);
+            flat_item(a, f, (unsigned)g0, (unsigned)(g1 - g0) * W, FlatGlobal{a.x + g0 * W});
+        }
+    }
+
+    // One thread per output: tensors of 2^31 rows or more.
     static __device__ void run_scalar(const Args &a, const Ctx &cx)
     {
         const int H = a.H, W = a.W, Ho = 2 * H, Wo = 2 * W;
@@ -278,12 +476,15 @@ struct BodyUpsample {
     static __device__ void run(const Args &a, const Ctx &cx)
     {
         if ((int64_t)a.P * a.H * a.W == 0) return;
-        if ((a.W & 3) == 0 && aligned16(a.x) && aligned16(a.y)) {
+        const bool flat = flat_range((int64_t)a.P * a.H, a.W, cx);
+        if (strips(a)) {
             if (a.W <= 128 && WarpRing::available(cx, 0) && run_ring(a, cx)) return;
-            run_vec(a, cx);
-        } else {
-            run_scalar(a, cx);
+        } else if (flat && flat_ring(a, cx)) {
+            return;
         }
+        if (a.W >= kStripCols && rows16(a)) run_vec(a, cx);
+        else if (flat) flat_global(a, cx);
+        else run_scalar(a, cx);
     }
 };
 
@@ -299,11 +500,21 @@ struct BodyMaxpool {
     static constexpr bool kRingItem = true;
     static constexpr unsigned kRingMinBytes = 4096;   // the stage: one item
 
-    // strips of whole rows (W <= 128, 16-byte rows) arrive as one bulk copy
+    // Which path: 16-byte rows of 64 values or more go to strips of whole
+    // rows (four columns a lane), the others to the flat path.  Strips leave
+    // lanes idle below 128 columns: 2^23 values in images of W = 8 / 16 /
+    // 32 / 40 / 56 / 64 columns took 74 / 43 / 28 / 25 / 22 / 21 us alone,
+    // the flat path 22 / 22 / 21 / 22 / 22 / 21 (at W = 112 strips 18, flat 21).
+    static constexpr int kStripCols = 64;
+    static __host__ __device__ bool strips(const Args &a)
+    {
+        return (a.W & 3) == 0 && a.W >= kStripCols && aligned16(a.x) && aligned16(a.y);
+    }
+    // a strip's rows (W <= 128) or a flat item's arrive as one bulk copy
     static __host__ bool uses_ring(const Args &a)
     {
-        return (int64_t)a.P * a.H * a.W > 0 && (a.W & 3) == 0 && a.W <= 128 && a.H >= 2 &&
-               aligned16(a.x) && aligned16(a.y);
+        if ((int64_t)a.P * a.H * a.W <= 0) return false;
+        return strips(a) ? a.W <= 128 && a.H >= 2 : aligned16(a.x) && 3u * a.W + kFlatPad <= kRingMinBytes / 4;
     }
 
     static __host__ size_t workspace_bytes(const Args &) { return 0; }
@@ -451,6 +662,104 @@ struct BodyMaxpool {
         return true;
     }
 
+    // One item of the flat path: its pixels are output pixels (W and H of f
+    // those of the output), get(0) is column 0 of the window centre of the
+    // item's first row, which is row oy0 of its plane.  The order of the
+    // maxima is the strips'; where W or an alignment rules strips out a NaN
+    // never wins (`clean`), as in one running maximum over the window.
+    template <class Get>
+    static __device__ __forceinline__ void flat_item(const Args &a, const FlatRows &f, unsigned oy0, unsigned n,
+                                                     float *y0, const Get &get)
+    {
+        const int W = a.W;
+        const unsigned H = (unsigned)a.H;
+        const bool clean = (a.W & 3) != 0 || !aligned16(a.x) || !aligned16(a.y);
+        const float ninf = -__int_as_float(0x7f800000);
+#pragma unroll 2
+        for (unsigned i = lane_id(); i < n; i += 32) {
+            const unsigned lr = f.row_of(i), ox = i - lr * f.W, t = oy0 + lr;
+            const unsigned p = f.plane_of(t), oy = t - p * f.H;
+            // input row 2*oy of plane p, counted from input row 2*oy0 of the
+            // item's first plane
+            const int cen = (int)(p * H + 2 * oy - 2 * oy0) * W + 2 * (int)ox;
+            const bool te = oy == 0, be = 2 * oy + 1 >= H, le = ox == 0, re = 2 * (int)ox + 1 >= W;
+            auto row3 = [&](int c, bool out) {
+                float l = get(c - 1, !out && !le);
+                const float x = get(c, !out);
+                const float r = get(c + 1, !out && !re);
+                if (le) l = ninf;
+                if (clean) l = mx(ninf, l);
+                const float h = mx(l, x);
+                return out ? ninf : re ? h : mx(h, r);
+            };
+            const float h0 = row3(cen - W, te), h1 = row3(cen, false), h2 = row3(cen + W, be);
+            __stcs(y0 + i, mx(mx(h0, h1), h2));
+        }
+    }
+
+    static __device__ bool flat_ring(const Args &a, const Ctx &cx)
+    {
+        const int H = a.H;
+        const unsigned W = (unsigned)a.W, Ho = (unsigned)(H - 1) / 2 + 1, Wo = (W - 1) / 2 + 1;
+        const int64_t rows = (int64_t)a.P * Ho, total = (int64_t)a.P * H * W;
+        const int nw = cx.nthreads >> 5;
+        const int64_t gw = (int64_t)cx.block * nw + (cx.tid >> 5), GW = (int64_t)cx.grid * nw;
+        const unsigned slots = min(cx.ring_stage, 4096u) / 4;
+        if (!aligned16(a.x) || 3 * W + kFlatPad > slots || !WarpRing::available(cx, 0)) return false;
+        FlatRows f;
+        // R output rows need at most 2R + 1 input rows
+        const unsigned rmax = ((slots - kFlatPad) / W - 1) / 2;
+        f.init(Wo, Ho, (unsigned)rows, min(rmax, FlatRows::kMaxValues / Wo), (unsigned)GW, 1);
+        WarpRing r;
+        r.init(cx, 0);
+        // input values of output rows [q0, q1), halo included
+        auto copy = [&](unsigned q0, unsigned q1, unsigned &p0, unsigned &oy0, int64_t &hi) {
+            p0 = q0 / Ho;
+            oy0 = q0 - p0 * Ho;
+            const unsigned p1 = (q1 - 1) / Ho, oy1 = q1 - 1 - p1 * Ho;
+            const int64_t lo = ((int64_t)p0 * H + 2 * (int64_t)oy0 - 1) * W - 1;
+            hi = ((int64_t)p1 * H + 2 * (int64_t)oy1 + 2) * W + 1;
+            return FlatCopy(lo, hi, total);
+        };
+        unsigned p0, oy0;
+        int64_t hi;
+        ring_stream(
+            r, gw, GW, f.items(),
+            [&](int st, int64_t it) {
+                const unsigned q0 = (unsigned)it * f.R, q1 = min(q0 + f.R, f.rows);
+                copy(q0, q1, p0, oy0, hi).fill(r, st, a.x);
+            },
+            [&](unsigned char *stage, int64_t it) {
+                const unsigned q0 = (unsigned)it * f.R, q1 = min(q0 + f.R, f.rows);
+                const FlatCopy k = copy(q0, q1, p0, oy0, hi);
+                k.patch(stage, a.x, hi, total, r.lane);
+                const int64_t first = ((int64_t)p0 * H + 2 * (int64_t)oy0) * W;
+                flat_item(a, f, oy0, (q1 - q0) * Wo, a.y + (int64_t)q0 * Wo,
+                          FlatStage{reinterpret_cast<const float *>(stage) + (first - k.base)});
+            });
+        r.finish();
+        return true;
+    }
+
+    // The same items without a ring.
+    static __device__ void flat_global(const Args &a, const Ctx &cx)
+    {
+        const int H = a.H;
+        const unsigned Ho = (unsigned)(H - 1) / 2 + 1, Wo = (unsigned)(a.W - 1) / 2 + 1;
+        const int64_t rows = (int64_t)a.P * Ho, W = a.W;
+        const int nw = cx.nthreads >> 5;
+        const int64_t gw = (int64_t)cx.block * nw + (cx.tid >> 5), GW = (int64_t)cx.grid * nw;
+        FlatRows f;
+        f.init(Wo, Ho, (unsigned)rows, max(1u, FlatRows::kMaxValues / Wo), (unsigned)GW, 1);
+        for (int64_t it = gw; it < f.items(); it += GW) {
+            const unsigned q0 = (unsigned)it * f.R, q1 = min(q0 + f.R, f.rows);
+            const unsigned p0 = q0 / Ho, oy0 = q0 - p0 * Ho;
+            flat_item(a, f, oy0, (q1 - q0) * Wo, a.y + (int64_t)q0 * Wo,
+                      FlatGlobal{a.x + ((int64_t)p0 * H + 2 * (int64_t)oy0) * W});
+        }
+    }
+
+    // One thread per output: tensors of 2^31 rows or more.
     static __device__ void run_scalar(const Args &a, const Ctx &cx)
     {
         const int H = a.H, W = a.W, Ho = (H - 1) / 2 + 1, Wo = (W - 1) / 2 + 1;
@@ -479,9 +788,11 @@ struct BodyMaxpool {
     static __device__ void run(const Args &a, const Ctx &cx)
     {
         if ((int64_t)a.P * a.H * a.W == 0) return;
-        if ((a.W & 3) == 0 && aligned16(a.x) && aligned16(a.y)) {
+        if (strips(a)) {
             if (a.W <= 128 && a.H >= 2 && WarpRing::available(cx, 0) && run_ring(a, cx)) return;
             run_vec(a, cx);
+        } else if (flat_range((int64_t)a.P * a.H, a.W, cx)) {
+            if (!flat_ring(a, cx)) flat_global(a, cx);
         } else {
             run_scalar(a, cx);
         }
@@ -498,16 +809,24 @@ struct BodyIm2col {
     static constexpr int kId = HF_BODY_IM2COL3;
     static constexpr int kBarriers = 0;
     // ring path: a stage holds an item's 14 rows and its two halo rows
-    // (rows of up to 64 floats)
+    // (rows of up to 64 floats), or at least three rows (the flat path)
     static constexpr int kRingRows = 14;
     static constexpr bool kRingItem = true;
     static constexpr unsigned kRingMinBytes = 4096;   // the stage: one item
-
-    // chunks of whole rows (W <= 64, 16-byte rows) arrive as one bulk copy
+    // Strips of 16-byte rows of 56 to 64 values, the flat path for all others.
+    // Both are at the write rate from four warps an SM on; with one warp an
+    // SM (an interval of a large schedule), where instructions count, 2^23
+    // values of W = 16 / 28 / 48 / 56 / 64 columns took strips 493 / 171 /
+    // 121 / 93 / 89 us and the flat path 105 / 105 / 109 / 101 / 108.
+    static constexpr int kStripCols = 56;
+    static __host__ __device__ bool rows16(const Args &a)
+    {
+        return (a.W & 3) == 0 && a.W <= 64 && aligned16(a.x) && aligned16(a.col);
+    }
     static __host__ bool uses_ring(const Args &a)
     {
-        return (int64_t)a.N * a.C * a.H * a.W > 0 && (a.W & 3) == 0 && a.W <= 64 && aligned16(a.x) &&
-               aligned16(a.col);
+        if ((int64_t)a.N * a.C * a.H * a.W <= 0) return false;
+        return (rows16(a) && a.W >= kStripCols) || (aligned16(a.x) && 3u * a.W + kFlatPad <= kRingMinBytes / 4);
     }
 
     static __host__ size_t workspace_bytes(const Args &) { return 0; }
@@ -676,6 +995,142 @@ struct BodyIm2col {
         return true;
     }
 
+    // One item of the flat path, VEC consecutive pixels per lane.  Shifted
+    // copy k of pixel i lies at k*HW + i of its plane's output, so a warp's
+    // stores are contiguous for any W; VEC == 4 (planes of 16-byte
+    // multiples, items that start on one) makes them 128-bit and reads
+    // three times six values for four pixels -- in one 128-bit and two
+    // 32-bit loads where the rows are 16-byte multiples too.
+    template <int VEC, class Get>
+    static __device__ __forceinline__ void flat_item(const Args &a, const FlatRows &f, unsigned g0, unsigned n,
+                                                     const Get &get)
+    {
+        const int W = (int)f.W;
+        const int64_t HW = (int64_t)f.H * W;
+        const unsigned p0 = g0 / f.H, r0 = g0 - p0 * f.H;
+        // output of the item's first pixel, copy 0, if its plane went on
+        float *o0 = a.col + ((int64_t)p0 * 9 * HW + (int64_t)r0 * W);
+        if constexpr (VEC == 4)
+            if ((W & 3) == 0) {   // the four pixels are of one row
+                for (unsigned i = 4 * lane_id(); i < n; i += 128) {
+                    const unsigned lr = f.row_of(i), t = r0 + lr, p = f.plane_of(t);
+                    const unsigned c = i - lr * f.W, r = t - p * f.H;
+                    const bool le = c == 0, re = c + 4 == f.W;
+                    float *o = o0 + ((int64_t)p * 8 * HW + i);
+#pragma unroll
+                    for (int ky = 0; ky < 3; ++ky) {
+                        const float *q = get.p + ((int)i + (ky - 1) * W);
+                        float4 m = *reinterpret_cast<const float4 *>(q);
+                        float L = q[-1], R = q[4];
+                        if ((ky == 0 && r == 0) || (ky == 2 && r == f.H - 1)) m = make_float4(0.f, 0.f, 0.f, 0.f), L = R = 0.f;
+                        if (le) L = 0.f;
+                        if (re) R = 0.f;
+                        emit(Row{m, L, R}, o + 3 * ky * HW, HW);
+                    }
+                }
+                return;
+            }
+        for (unsigned i = VEC * lane_id(); i < n; i += 32 * VEC) {
+            const unsigned lr = f.row_of(i), t = r0 + lr;
+            const unsigned p = f.plane_of(t);
+            unsigned c = i - lr * f.W, r = t - p * f.H;
+            bool le[VEC], re[VEC], te[VEC], be[VEC];
+#pragma unroll
+            for (int v = 0; v < VEC; ++v) {
+                le[v] = c == 0;
+                re[v] = c == f.W - 1;
+                te[v] = r == 0;
+                be[v] = r == f.H - 1;
+                if (++c == f.W) c = 0, ++r;   // planes end on multiples of VEC
+            }
+            float *o = o0 + ((int64_t)p * 8 * HW + i);
+            // not unrolled: unrolled it took eight registers more in the
+            // fused kernels, which cost them blocks of 640 threads
+#pragma unroll 1
+            for (int ky = 0; ky < 3; ++ky) {
+                const int off = (int)i + (ky - 1) * W;
+                float q[VEC + 2], w[3][VEC];
+#pragma unroll
+                for (int v = 0; v < VEC + 2; ++v) {
+                    // the value at off + v - 1 is read by pixel v - 1 + {1, 0, -1}
+                    // (for global loads: by one that is inside)
+                    bool ok = false;
+#pragma unroll
+                    for (int kx = 0; kx < 3; ++kx) {
+                        const int px = v - kx;
+                        if (px < 0 || px >= VEC) continue;
+                        const bool out = (ky == 0 && te[px]) || (ky == 2 && be[px]) || (kx == 0 && le[px]) ||
+                                         (kx == 2 && re[px]);
+                        ok = ok || !out;
+                    }
+                    q[v] = get(off + v - 1, ok);
+                }
+#pragma unroll
+                for (int v = 0; v < VEC; ++v) {
+                    const bool out = (ky == 0 && te[v]) || (ky == 2 && be[v]);
+                    w[0][v] = out || le[v] ? 0.f : q[v];
+                    w[1][v] = out ? 0.f : q[v + 1];
+                    w[2][v] = out || re[v] ? 0.f : q[v + 2];
+                }
+#pragma unroll
+                for (int kx = 0; kx < 3; ++kx) {
+                    float *d = o + (3 * ky + kx) * HW;
+                    if (VEC == 4) stcs4(d, make_float4(w[kx][0], w[kx][1 % VEC], w[kx][2 % VEC], w[kx][3 % VEC]));
+                    else __stcs(d, w[kx][0]);
+                }
+            }
+        }
+    }
+
+    template <int VEC>
+    static __device__ __forceinline__ bool flat_ring(const Args &a, const Ctx &cx)
+    {
+        const int64_t rows = (int64_t)a.N * a.C * a.H, total = rows * a.W;
+        const int nw = cx.nthreads >> 5;
+        const int64_t gw = (int64_t)cx.block * nw + (cx.tid >> 5), GW = (int64_t)cx.grid * nw;
+        const unsigned W = (unsigned)a.W, slots = min(cx.ring_stage, 4096u) / 4;
+        // items of whole 16-byte multiples
+        const unsigned mult = VEC == 1 || (W & 3) == 0 ? 1u : (W & 1) ? 4u : 2u;
+        if (!aligned16(a.x) || (mult + 2) * W + kFlatPad > slots || !WarpRing::available(cx, 0)) return false;
+        unsigned rmax = min((slots - kFlatPad) / W - 2, FlatRows::kMaxValues / W);
+        rmax -= rmax % mult;
+        FlatRows f;
+        f.init(W, a.H, (unsigned)rows, rmax, (unsigned)GW, mult);
+        WarpRing r;
+        r.init(cx, 0);
+        auto copy = [&](int64_t it) {
+            const int64_t g0 = it * f.R;
+            return FlatCopy((g0 - 1) * W - 1, (min(g0 + (int64_t)f.R, rows) + 1) * W + 1, total);
+        };
+        ring_stream(
+            r, gw, GW, f.items(), [&](int st, int64_t it) { copy(it).fill(r, st, a.x); },
+            [&](unsigned char *stage, int64_t it) {
+                const int64_t g0 = it * f.R, g1 = min(g0 + (int64_t)f.R, rows);
+                const FlatCopy k = copy(it);
+                k.patch(stage, a.x, (g1 + 1) * W + 1, total, r.lane);
+                flat_item<VEC>(a, f, (unsigned)g0, (unsigned)(g1 - g0) * W,
+                               FlatStage{reinterpret_cast<const float *>(stage) + (g0 * W - k.base)});
+            });
+        r.finish();
+        return true;
+    }
+
+    // The same items, one pixel per lane, without a ring.
+    static __device__ void flat_global(const Args &a, const Ctx &cx)
+    {
+        const int64_t rows = (int64_t)a.N * a.C * a.H;
+        const int nw = cx.nthreads >> 5;
+        const int64_t gw = (int64_t)cx.block * nw + (cx.tid >> 5), GW = (int64_t)cx.grid * nw;
+        const unsigned W = (unsigned)a.W;
+        FlatRows f;
+        f.init(W, a.H, (unsigned)rows, max(1u, FlatRows::kMaxValues / W), (unsigned)GW, 1);
+        for (int64_t it = gw; it < f.items(); it += GW) {
+            const int64_t g0 = it * f.R, g1 = min(g0 + (int64_t)f.R, rows);
+            flat_item<1>(a, f, (unsigned)g0, (unsigned)(g1 - g0) * W, FlatGlobal{a.x + g0 * W});
+        }
+    }
+
+    // One thread per output: tensors of 2^31 rows or more.
     static __device__ void run_scalar(const Args &a, const Ctx &cx)
     {
         const int H = a.H, W = a.W;
@@ -698,12 +1153,17 @@ struct BodyIm2col {
     static __device__ void run(const Args &a, const Ctx &cx)
     {
         if ((int64_t)a.N * a.C * a.H * a.W == 0) return;
-        if ((a.W & 3) == 0 && a.W <= 64 && aligned16(a.x) && aligned16(a.col)) {
+        const bool flat = flat_range((int64_t)a.N * a.C * a.H, a.W, cx);
+        if (rows16(a) && a.W >= kStripCols) {
             if (WarpRing::available(cx, 0) && run_ring(a, cx)) return;
-            run_vec(a, cx);
-        } else {
-            run_scalar(a, cx);
+        } else if (flat) {
+            const bool v4 = a.W >= 4 && ((int64_t)a.H * a.W & 3) == 0 && aligned16(a.col);
+            if (v4 && flat_ring<4>(a, cx)) return;
+            if (flat_ring<1>(a, cx)) return;
         }
+        if (rows16(a)) run_vec(a, cx);
+        else if (flat) flat_global(a, cx);
+        else run_scalar(a, cx);
     }
 };
 
