@@ -673,7 +673,7 @@ hf_status hf_cost_model_set(const float *params, int n_models, float mu, float s
 hf_status hf_mlp_forward(const float *params, const float *X, int n, float *y, void *stream);
 
 /* Trains params in place with Adam on the mean squared error, all `steps`
- * steps in one kernel launch (one thread block): step s uses the batch rows
+ * steps in one kernel launch (one cluster of eight thread blocks): step s uses the batch rows
  * idx[s*batch .. s*batch + batch) of X[.][24] / Y[.] (batch <= 64); adam_m
  * and adam_v are the first and second moment arrays (device, HF_MLP_NPARAMS
  * each, zero for a fresh run); t0 is the number of Adam steps already taken.

@@ -11,13 +11,8 @@
 // second layer's (transposed) in shared memory, and the output is a warp
 // butterfly sum.
 //
-// k_mlp_train runs a whole training run in ONE persistent block: for each
-// step it gathers a minibatch (rows idx[step*B .. step*B+B)), runs the
-// forward pass, back-propagates the mean squared error, and applies Adam
-// (Kingma & Ba) to parameters held in shared memory.  Every activation and
-// gradient lives in shared memory with padded rows (stride 65 / 25) so that
-// lanes that walk samples hit distinct banks; every sum has a fixed order,
-// so a run is deterministic.
+// k_mlp_train runs a whole training run in one launch of one cluster of eight
+// blocks; see its comment.
 #include <cmath>
 
 #include "kernels.cuh"
@@ -31,8 +26,6 @@ namespace {
 constexpr int IN = 24, HD = 64, NP = 5825;
 constexpr int OW1 = 0, OB1 = 1536, OW2 = 1600, OB2 = 5696, OW3 = 5760, OB3 = 5824;
 constexpr int kMaxBatch = 64;
-constexpr int kTrainThreads = 512;
-constexpr int SX = IN + 1, SH = HD + 1;   // padded row strides
 
 __global__ void __launch_bounds__(256) k_mlp_forward(const float *__restrict__ P,
                                                      const float *__restrict__ X, int n,
@@ -82,139 +75,353 @@ __global__ void __launch_bounds__(256) k_mlp_forward(const float *__restrict__ P
     }
 }
 
+// ------------------------------------------------------------------ training
+// One cluster of kCl blocks runs every step: gather, forward, backward (mean
+// squared error) and Adam (Kingma & Ba).  Block r owns hidden units
+// 8r .. 8r+7 of both layers: their rows of W1 and W2, the same columns of W2
+// (a copy for the backward pass), their biases, their w3, and the moments of
+// all of them, which stay in the registers of the threads that update them.
+// Activations are kept transposed ([unit][sample]) so that every product is
+// an outer-product tile of 128-bit shared loads:
+//   columns<K>  out[u][s..s+3] += W[u][k] * A[k][s..s+3], lanes = 8 units x 4
+//               groups of four samples: 5 loads per 16 multiply-adds
+//               (forward layers, and the backward pass through W2)
+//   gradient    g[u][i] += D[u][s] * A[i][s], lanes = 8 units x 4 inputs
+// Blocks exchange the two activation layers through distributed shared
+// memory: each writes its units' rows into all blocks, two cluster barriers a
+// step; updated columns of W2 and w3 travel with the next step's first one.
+// What a slower block may still read (H1, the W2 columns, w3) is double
+// buffered: a block past a step's barriers knows that every other one has
+// finished the step before.  Two warps gather the next step's batch meanwhile.
+//
+// The bound is latency: a step is a chain of five products of 24 to 64
+// dependent multiply-adds, two cluster barriers and five block barriers, and
+// about 1000 cycles of multiply-add issue per block.  A single block with
+// one output per thread and both operands from shared memory (10 block
+// barriers, its load pipe 65 % busy) took 37.3 us a step at batch 64;
+// this takes 8.1 us, with the same bits.  Every sum keeps one fixed order (inputs or samples
+// ascending), so a run is deterministic; samples past the batch count as zero.
+constexpr int kCl = 8, kU = HD / kCl;    // blocks of the cluster, units per block
+constexpr int kWarps = 11, kTrainThreads = 32 * kWarps;
+constexpr int S = 68;                    // row stride of sample rows: 8 rows hit distinct banks
+constexpr int S1 = 28;                   // of W1's rows
 struct TrainSmem {
-    float P[NP], M[NP], V[NP], G[NP];
-    float X[kMaxBatch * SX];
-    float H1[kMaxBatch * SH];
-    float H2[kMaxBatch * SH];   // becomes D2 after the output layer's gradient
-    float D1[kMaxBatch * SH];
-    float Y[kMaxBatch], dY[kMaxBatch];
+    float Xt[2][IN][S];      // batch, transposed, of this and the next step
+    float H1[2][HD][S];      // all units, written by their owners
+    float H2[HD][S];
+    float D2[HD][S];         // error at layer 2, all units
+    float D1[kU][S];         // error at layer 1, own units
+    float W2[kU][S];         // own rows (own units over all inputs)
+    float W2c[2][kU][S];     // own columns: W2c[i][j] = W2[j][8r + i]
+    float W1[kU][S1];
+    float w3[2][HD];
+    float Y[2][HD], dY[HD], e2[HD], ones[HD];
+    float b1[kU], b2[kU], b3[2];
+    float c[2][2];           // Adam's bias corrections of this and the next step
+};
+static_assert(HD == 64 && kMaxBatch == 64 && kU == 8, "lane layout of the training kernel");
+
+__device__ __forceinline__ unsigned cluster_rank()
+{
+    unsigned r;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+// Every thread of the cluster arrives and waits (a hardware barrier over
+// co-scheduled blocks); shared-memory writes before it, remote ones too, are
+// visible after it.
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// address of `p`'s counterpart in block `rank` of the cluster
+__device__ __forceinline__ unsigned remote(const void *p, int rank)
+{
+    unsigned a;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((unsigned)__cvta_generic_to_shared(p)), "r"(rank));
+    return a;
+}
+__device__ __forceinline__ void put(unsigned addr, float v)
+{
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
+}
+__device__ __forceinline__ void put4(unsigned addr, float4 v)
+{
+    asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w)
+                 : "memory");
+}
+__device__ __forceinline__ float4 at4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
+__device__ __forceinline__ float part(const float4 &v, int i) { return i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w; }
+
+// acc[0..3] += sum over k (ascending) of w[k] * A[k][0..3]; A's rows S apart
+template <int K>
+__device__ __forceinline__ void columns(const float *w, const float *A, float4 &acc)
+{
+#pragma unroll 4
+    for (int k = 0; k < K; k += 4) {
+        const float4 w4 = at4(w + k);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const float4 a = at4(A + (k + j) * S);
+            const float wk = part(w4, j);
+            acc.x = __fmaf_rn(wk, a.x, acc.x);
+            acc.y = __fmaf_rn(wk, a.y, acc.y);
+            acc.z = __fmaf_rn(wk, a.z, acc.z);
+            acc.w = __fmaf_rn(wk, a.w, acc.w);
+        }
+    }
+}
+// g[v] += sum over s < n (ascending, n a multiple of 4) of d[s] * A_v[s],
+// the rows A_v 4 * S apart
+template <int N>
+__device__ __forceinline__ void gradient(const float *d, const float *A, int n, float (&g)[N])
+{
+#pragma unroll 4
+    for (int s = 0; s < n; s += 4) {
+        const float4 d4 = at4(d + s);
+#pragma unroll
+        for (int v = 0; v < N; ++v) {
+            const float4 a = at4(A + 4 * v * S + s);
+            g[v] = __fmaf_rn(d4.x, a.x, g[v]);
+            g[v] = __fmaf_rn(d4.y, a.y, g[v]);
+            g[v] = __fmaf_rn(d4.z, a.z, g[v]);
+            g[v] = __fmaf_rn(d4.w, a.w, g[v]);
+        }
+    }
+}
+
+// The moments' sums are one fused multiply-add each, spelled out so that
+// every use rounds alike.
+struct Adam {
+    float lr, beta1, beta2, eps;
+    __device__ __forceinline__ float step(float p, float &M, float &V, float g, const float *c) const
+    {
+        const float m = __fmaf_rn(1.f - beta1, g, beta1 * M);
+        const float v = __fmaf_rn((1.f - beta2) * g, g, beta2 * V);
+        M = m;
+        V = v;
+        return p - lr * (m / c[0]) / (sqrtf(v / c[1]) + eps);
+    }
 };
 
-__global__ void __launch_bounds__(kTrainThreads) k_mlp_train(
-    float *__restrict__ Pg, float *__restrict__ Mg, float *__restrict__ Vg,
-    const float *__restrict__ X, const float *__restrict__ Y, const int *__restrict__ idx,
-    int steps, int B, float lr, float beta1, float beta2, float eps, int t0,
-    float *__restrict__ loss_out, float *__restrict__ grad_out)
+__global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kTrainThreads) k_mlp_train(
+    float *__restrict__ Pg, float *__restrict__ Mg, float *__restrict__ Vg, const float *__restrict__ X,
+    const float *__restrict__ Y, const int *__restrict__ idx, int steps, int B, float lr, float beta1, float beta2,
+    float eps, int t0, float *__restrict__ loss_out, float *__restrict__ grad_out)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    TrainSmem &S = *reinterpret_cast<TrainSmem *>(smem_raw);
-    const int tid = threadIdx.x, T = blockDim.x;
-    for (int p = tid; p < NP; p += T) {
-        S.P[p] = Pg[p];
-        S.M[p] = Mg[p];
-        S.V[p] = Vg[p];
-    }
-    __syncthreads();
+    TrainSmem &T = *reinterpret_cast<TrainSmem *>(smem_raw);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int r = (int)cluster_rank(), j0 = kU * r;
+    const int n = (B + 3) / 4 * 4;            // samples of the padded batch
     const float invB = 1.0f / (float)B;
-    for (int step = 0; step < steps; ++step) {
-        // gather the minibatch
-        const int *rows = idx + (int64_t)step * B;
-        for (int e = tid; e < B * IN; e += T) {
-            const int s = e / IN, k = e % IN;
-            S.X[s * SX + k] = X[(int64_t)rows[s] * IN + k];
+    const Adam adam{lr, beta1, beta2, eps};
+
+    // parameters of this block's units (rows past n of the sample buffers are
+    // never read)
+    for (int e = tid; e < kU * IN; e += kTrainThreads) T.W1[e / IN][e % IN] = Pg[OW1 + j0 * IN + e];
+    for (int e = tid; e < kU * HD; e += kTrainThreads) {
+        T.W2[e / HD][e % HD] = Pg[OW2 + j0 * HD + e];
+        T.W2c[0][e % kU][e / kU] = Pg[OW2 + e / kU * HD + j0 + e % kU];
+    }
+    for (int e = tid; e < HD; e += kTrainThreads) {
+        T.w3[0][e] = Pg[OW3 + e];
+        T.ones[e] = 1.f;
+        if (e < kU) T.b1[e] = Pg[OB1 + j0 + e], T.b2[e] = Pg[OB2 + j0 + e];
+        if (e == 0) T.b3[0] = Pg[OB3];
+    }
+    // Who updates what: warps 0-3 four elements of W2 each thread; tid < 192
+    // one of W1; warp 8 the vectors (lanes 0-7 w3, 8-15 b2, 16 b3; then
+    // lanes 0-7 b1).
+    const int u = lane >> 2, q = lane & 3;
+    const int p_w2 = OW2 + (j0 + u) * HD + 16 * warp + q;   // + 4 * v
+    const int p_w1 = OW1 + j0 * IN + tid;
+    const int p_vec = lane < 8 ? OW3 + j0 + lane : lane < 16 ? OB2 + j0 + lane - 8 : OB3;
+    const int p_b1 = OB1 + j0 + (lane & 7);
+    float m2[4], v2[4], m1 = 0.f, v1 = 0.f, mv = 0.f, vv = 0.f;
+    if (warp < 4)
+#pragma unroll
+        for (int v = 0; v < 4; ++v) m2[v] = Mg[p_w2 + 4 * v], v2[v] = Vg[p_w2 + 4 * v];
+    if (tid < kU * IN) m1 = Mg[p_w1], v1 = Vg[p_w1];
+    if (warp == 8) {
+        mv = Mg[p_vec], vv = Vg[p_vec];
+        m1 = Mg[p_b1], v1 = Vg[p_b1];
+    }
+    // Warps 9 and 10, a lane per sample: the batch of step t is loaded into
+    // registers a step ahead and stored into buffer t & 1 when its loads
+    // have had two layers' time; its row number is loaded a step earlier still.
+    const int sample = 32 * (warp - 9) + lane;
+    float x[IN], y = 0.f;
+    int row = 0;
+    auto fetch_row = [&](int t) { row = sample < B && t < steps ? idx[(int64_t)t * B + sample] : 0; };
+    auto fetch = [&]() {
+#pragma unroll
+        for (int k = 0; k < IN; ++k) x[k] = sample < B ? __ldg(X + (int64_t)row * IN + k) : 0.f;
+        y = sample < B ? __ldg(Y + row) : 0.f;
+    };
+    auto stash = [&](int t) {
+        if (sample < n) {
+#pragma unroll
+            for (int k = 0; k < IN; ++k) T.Xt[t & 1][k][sample] = x[k];
+            T.Y[t & 1][sample] = y;
         }
-        for (int s = tid; s < B; s += T) S.Y[s] = Y[rows[s]];
+        if (sample == 0) {
+            const float tf = (float)(t0 + t + 1);
+            T.c[t & 1][0] = 1.f - powf(beta1, tf);
+            T.c[t & 1][1] = 1.f - powf(beta2, tf);
+        }
+    };
+    if (warp >= 9) {
+        fetch_row(0);
+        fetch();
+        stash(0);
+        fetch_row(1);
+    }
+    cluster_sync();   // every block has started; its buffers are ready
+
+    const int s4 = 16 * (warp & 3) + 4 * q;   // first sample of this lane's four
+    for (int t = 0; t < steps; ++t) {
+        const int cur = t & 1, nxt = cur ^ 1;
+        const float *c = T.c[cur];
+        if (warp >= 9 && t + 1 < steps) {
+            fetch();
+            fetch_row(t + 2);
+        }
+        // H1 = relu(X W1^T + b1), own units, into every block
+        if (warp < 4 && s4 < n) {
+            const float b = T.b1[u];
+            float4 a = make_float4(b, b, b, b);
+            columns<IN>(T.W1[u], &T.Xt[cur][0][s4], a);
+            a = make_float4(fmaxf(a.x, 0.f), fmaxf(a.y, 0.f), fmaxf(a.z, 0.f), fmaxf(a.w, 0.f));
+#pragma unroll
+            for (int k = 0; k < kCl; ++k) put4(remote(&T.H1[cur][j0 + u][s4], k), a);
+        }
+        cluster_sync();
+        // H2 = relu(H1 W2^T + b2), own units, into every block
+        if (warp < 4 && s4 < n) {
+            const float b = T.b2[u];
+            float4 a = make_float4(b, b, b, b);
+            columns<HD>(T.W2[u], &T.H1[cur][0][s4], a);
+            a = make_float4(fmaxf(a.x, 0.f), fmaxf(a.y, 0.f), fmaxf(a.z, 0.f), fmaxf(a.w, 0.f));
+#pragma unroll
+            for (int k = 0; k < kCl; ++k) put4(remote(&T.H2[j0 + u][s4], k), a);
+        }
+        cluster_sync();
+        // output, error and dL/dy of every sample, in every block
+        if (tid < n) {
+            float a = T.b3[0];
+#pragma unroll 4
+            for (int j = 0; j < HD; j += 4) {
+                const float4 w = at4(T.w3[cur] + j);
+                a = __fmaf_rn(w.x, T.H2[j][tid], a);
+                a = __fmaf_rn(w.y, T.H2[j + 1][tid], a);
+                a = __fmaf_rn(w.z, T.H2[j + 2][tid], a);
+                a = __fmaf_rn(w.w, T.H2[j + 3][tid], a);
+            }
+            const float e = tid < B ? a - T.Y[cur][tid] : 0.f;
+            T.dY[tid] = 2.f * e * invB;
+            T.e2[tid] = e * e;
+        }
         __syncthreads();
-        // H1 = relu(X W1^T + b1); lanes walk samples
-        for (int o = tid; o < B * HD; o += T) {
-            const int j = o / B, s = o % B;
-            float a = S.P[OB1 + j];
-            for (int k = 0; k < IN; ++k) a = __fmaf_rn(S.P[OW1 + j * IN + k], S.X[s * SX + k], a);
-            S.H1[s * SH + j] = fmaxf(a, 0.f);
+        // D2 = dY w3^T masked by the ReLU, all units
+        for (int e = tid; e < HD * (n / 4); e += kTrainThreads) {
+            const int j = e / (n / 4), s = 4 * (e - j * (n / 4));
+            const float w = T.w3[cur][j];
+            const float4 h = at4(&T.H2[j][s]), d = at4(T.dY + s);
+            *reinterpret_cast<float4 *>(&T.D2[j][s]) =
+                make_float4(h.x > 0.f ? d.x * w : 0.f, h.y > 0.f ? d.y * w : 0.f, h.z > 0.f ? d.z * w : 0.f,
+                            h.w > 0.f ? d.w * w : 0.f);
         }
         __syncthreads();
-        // H2 = relu(H1 W2^T + b2)
-        for (int o = tid; o < B * HD; o += T) {
-            const int j = o / B, s = o % B;
-            float a = S.P[OB2 + j];
-            for (int i = 0; i < HD; ++i) a = __fmaf_rn(S.P[OW2 + j * HD + i], S.H1[s * SH + i], a);
-            S.H2[s * SH + j] = fmaxf(a, 0.f);
+        if (warp < 4) {
+            // W2's own rows: gW2[j][i] = sum_s D2[s][j] H1[s][i]
+            float g[4] = {0.f, 0.f, 0.f, 0.f};
+            const int i0 = 16 * warp + q;
+            gradient<4>(T.D2[j0 + u], T.H1[cur][i0], n, g);
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                const int i = i0 + 4 * v;
+                if (grad_out && t == 0) grad_out[p_w2 + 4 * v] = g[v];
+                const float w = adam.step(T.W2[u][i], m2[v], v2[v], g[v], c);
+                T.W2[u][i] = w;
+                put(remote(&T.W2c[nxt][i & 7][j0 + u], i >> 3), w);   // unit i's block
+            }
+        } else if (warp < 8) {
+            // D1[s][i] = (sum_j D2[s][j] W2[j][i]) masked by the ReLU, own units
+            if (s4 < n) {
+                float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+                columns<HD>(T.W2c[cur][u], &T.D2[0][s4], a);
+                const float4 h = at4(&T.H1[cur][j0 + u][s4]);
+                *reinterpret_cast<float4 *>(&T.D1[u][s4]) =
+                    make_float4(h.x > 0.f ? a.x : 0.f, h.y > 0.f ? a.y : 0.f, h.z > 0.f ? a.z : 0.f,
+                                h.w > 0.f ? a.w : 0.f);
+            }
+        } else if (warp == 8) {
+            // sums over the samples: gw3 and gb2 of the own units, gb3, loss
+            if (lane < 18) {
+                const float *d = lane < 8 ? T.dY : T.ones;
+                const float *a = lane < 8 ? T.H2[j0 + lane] : lane < 16 ? T.D2[j0 + lane - 8] : lane == 16 ? T.dY : T.e2;
+                float g[1] = {0.f};
+                gradient<1>(d, a, n, g);
+                if (lane == 17) {
+                    if (r == 0 && loss_out) loss_out[t] = g[0] * invB;
+                } else {
+                    if (grad_out && t == 0 && (lane < 16 || r == 0)) grad_out[p_vec] = g[0];
+                    const float old = lane < 8 ? T.w3[cur][j0 + lane] : lane < 16 ? T.b2[lane - 8] : T.b3[0];
+                    const float w = adam.step(old, mv, vv, g[0], c);
+                    if (lane < 8) {
+#pragma unroll
+                        for (int k = 0; k < kCl; ++k) put(remote(&T.w3[nxt][j0 + lane], k), w);
+                    } else if (lane < 16) {
+                        T.b2[lane - 8] = w;
+                    } else {
+                        T.b3[0] = w;   // the same bits in every block
+                    }
+                }
+            }
+        } else if (t + 1 < steps) {
+            stash(t + 1);
         }
         __syncthreads();
-        // output, error and dL/dy (mean squared error)
-        for (int s = tid; s < B; s += T) {
-            float a = S.P[OB3];
-            for (int j = 0; j < HD; ++j) a = __fmaf_rn(S.P[OW3 + j], S.H2[s * SH + j], a);
-            const float e = a - S.Y[s];
-            S.dY[s] = 2.f * e * invB;
-            S.D1[s] = e * e;   // scratch for the loss
-        }
-        __syncthreads();
-        if (tid == 0 && loss_out) {
-            float l = 0.f;
-            for (int s = 0; s < B; ++s) l += S.D1[s];
-            loss_out[step] = l * invB;
-        }
-        // gradients of the output layer
-        for (int j = tid; j <= HD; j += T) {
-            float g = 0.f;
-            if (j < HD)
-                for (int s = 0; s < B; ++s) g = __fmaf_rn(S.dY[s], S.H2[s * SH + j], g);
-            else
-                for (int s = 0; s < B; ++s) g += S.dY[s];
-            S.G[j < HD ? OW3 + j : OB3] = g;
-        }
-        __syncthreads();
-        // D2 = dY w3^T masked by the ReLU, in place of H2
-        for (int o = tid; o < B * HD; o += T) {
-            const int j = o / B, s = o % B;
-            const float h = S.H2[s * SH + j];
-            S.H2[s * SH + j] = h > 0.f ? S.dY[s] * S.P[OW3 + j] : 0.f;
-        }
-        __syncthreads();
-        // gW2[j][i] = sum_s D2[s][j] H1[s][i]; gb2[j] = sum_s D2[s][j]
-        for (int o = tid; o < HD * HD; o += T) {
-            const int j = o / HD, i = o % HD;
-            float g = 0.f;
-            for (int s = 0; s < B; ++s) g = __fmaf_rn(S.H2[s * SH + j], S.H1[s * SH + i], g);
-            S.G[OW2 + o] = g;
-        }
-        for (int j = tid; j < HD; j += T) {
-            float g = 0.f;
-            for (int s = 0; s < B; ++s) g += S.H2[s * SH + j];
-            S.G[OB2 + j] = g;
-        }
-        // D1[s][i] = (sum_j D2[s][j] W2[j][i]) masked by the ReLU
-        for (int o = tid; o < B * HD; o += T) {
-            const int i = o / B, s = o % B;
-            float a = 0.f;
-            for (int j = 0; j < HD; ++j) a = __fmaf_rn(S.H2[s * SH + j], S.P[OW2 + j * HD + i], a);
-            S.D1[s * SH + i] = S.H1[s * SH + i] > 0.f ? a : 0.f;
-        }
-        __syncthreads();
-        // gW1[j][k] = sum_s D1[s][j] X[s][k]; gb1[j] = sum_s D1[s][j]
-        for (int o = tid; o < HD * IN; o += T) {
-            const int j = o / IN, k = o % IN;
-            float g = 0.f;
-            for (int s = 0; s < B; ++s) g = __fmaf_rn(S.D1[s * SH + j], S.X[s * SX + k], g);
-            S.G[OW1 + o] = g;
-        }
-        for (int j = tid; j < HD; j += T) {
-            float g = 0.f;
-            for (int s = 0; s < B; ++s) g += S.D1[s * SH + j];
-            S.G[OB1 + j] = g;
-        }
-        __syncthreads();
-        if (grad_out && step == 0)
-            for (int p = tid; p < NP; p += T) grad_out[p] = S.G[p];
-        // Adam
-        const int t = t0 + step + 1;
-        const float c1 = 1.f - powf(beta1, (float)t), c2 = 1.f - powf(beta2, (float)t);
-        for (int p = tid; p < NP; p += T) {
-            const float g = S.G[p];
-            const float m = beta1 * S.M[p] + (1.f - beta1) * g;
-            const float v = beta2 * S.V[p] + (1.f - beta2) * g * g;
-            S.M[p] = m;
-            S.V[p] = v;
-            S.P[p] -= lr * (m / c1) / (sqrtf(v / c2) + eps);
+        // W1's own rows: gW1[j][k] = sum_s D1[s][j] X[s][k]
+        if (tid < kU * IN) {
+            const int j = tid / IN, k = tid - j * IN;
+            float g[1] = {0.f};
+            gradient<1>(T.D1[j], T.Xt[cur][k], n, g);
+            if (grad_out && t == 0) grad_out[p_w1] = g[0];
+            T.W1[j][k] = adam.step(T.W1[j][k], m1, v1, g[0], c);
+        } else if (warp == 8 && lane < 8) {
+            float g[1] = {0.f};
+            gradient<1>(T.ones, T.D1[lane], n, g);
+            if (grad_out && t == 0) grad_out[p_b1] = g[0];
+            T.b1[lane] = adam.step(T.b1[lane], m1, v1, g[0], c);
         }
         __syncthreads();
     }
-    for (int p = tid; p < NP; p += T) {
-        Pg[p] = S.P[p];
-        Mg[p] = S.M[p];
-        Vg[p] = S.V[p];
+    cluster_sync();   // no block leaves while others may write to it
+    if (warp < 4)
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            Pg[p_w2 + 4 * v] = T.W2[u][16 * warp + q + 4 * v];
+            Mg[p_w2 + 4 * v] = m2[v];
+            Vg[p_w2 + 4 * v] = v2[v];
+        }
+    if (tid < kU * IN) {
+        Pg[p_w1] = T.W1[tid / IN][tid % IN];
+        Mg[p_w1] = m1;
+        Vg[p_w1] = v1;
+    }
+    if (warp == 8) {
+        if (lane < 16 || (lane == 16 && r == 0)) {
+            Pg[p_vec] = lane < 8 ? T.w3[steps & 1][j0 + lane] : lane < 16 ? T.b2[lane - 8] : T.b3[0];
+            Mg[p_vec] = mv;
+            Vg[p_vec] = vv;
+        }
+        if (lane < 8) {
+            Pg[p_b1] = T.b1[lane];
+            Mg[p_b1] = m1;
+            Vg[p_b1] = v1;
+        }
     }
 }
 
@@ -246,7 +453,7 @@ hf_status hf_mlp_train(float *params, float *adam_m, float *adam_v, const float 
     const size_t smem = sizeof(TrainSmem);
     cudaError_t e = cudaFuncSetAttribute(k_mlp_train, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return hf::set_last_error(HF_ERR_CUDA, cudaGetErrorString(e));
-    k_mlp_train<<<1, kTrainThreads, smem, static_cast<cudaStream_t>(stream)>>>(
+    k_mlp_train<<<kCl, kTrainThreads, smem, static_cast<cudaStream_t>(stream)>>>(
         params, adam_m, adam_v, X, Y, idx, steps, batch, lr, beta1, beta2, eps, t0, loss_out, grad_out);
     e = cudaGetLastError();
     return e == cudaSuccess ? HF_OK : hf::set_last_error(HF_ERR_CUDA, cudaGetErrorString(e));
