@@ -6,10 +6,8 @@
 //   W1[64][24] @0, b1[64] @1536, W2[64][64] @1600, b2[64] @5696,
 //   w3[64] @5760, b3 @5824                                  (5825 values)
 //
-// k_mlp_forward scores samples grid-wide: one warp per sample, lane j owns
-// hidden units j and j+32, the first layer's weights sit in registers, the
-// second layer's (transposed) in shared memory, and the output is a warp
-// butterfly sum.
+// k_mlp_forward scores samples grid-wide, in tiles of 32 samples; see its
+// comment.
 //
 // k_mlp_train runs a whole training run in one launch of one cluster of eight
 // blocks; see its comment.
@@ -27,51 +25,134 @@ constexpr int IN = 24, HD = 64, NP = 5825;
 constexpr int OW1 = 0, OB1 = 1536, OW2 = 1600, OB2 = 5696, OW3 = 5760, OB3 = 5824;
 constexpr int kMaxBatch = 64;
 
-__global__ void __launch_bounds__(256) k_mlp_forward(const float *__restrict__ P,
-                                                     const float *__restrict__ X, int n,
-                                                     float *__restrict__ y)
+// ------------------------------------------------------------------ forward
+__device__ __forceinline__ float4 at4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
+__device__ __forceinline__ float part(const float4 &v, int i) { return i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w; }
+
+// A tile is 32 samples and belongs to two warps: lane = four samples (q) and
+// eight units ug, ug + 8, ..., ug + 56, so that twelve 128-bit shared loads
+// (four of activations, eight of weights) feed 128 multiply-adds.  The
+// weights are staged once per block and the activations stay transposed
+// ([unit][sample]); rows of 68, 28 and 36 values keep the loads free of
+// bank conflicts.  A block has kSlots tiles in work; tiles go to blocks
+// first and slots second, so few samples spread over the SMs.
+//
+// The bound is the shared-load pipe (an LDS.128 takes it four cycles
+// whatever it broadcasts): about 2100 cycles a tile against 1400 of
+// multiply-adds on four schedulers.  One warp per sample, with two 32-bit
+// weight loads and a shuffle per two multiply-adds and a transpose of W2
+// with 32-way bank conflicts in every block, took 32.8 us for 16086 samples
+// and 7.4 for 100; this takes 7.1 and 4.6 us (most of the latter is the
+// weights' way into shared memory: 7.3 us before all of a thread's loads
+// were in flight at once).  Both sum in the same order: the same bits.
+constexpr int kSlots = 2, kTile = 32, FS = 36;   // FS: row stride of a tile's rows
+struct ForwardSmem {
+    float W2[HD][68];
+    float W1[HD][28];
+    float A[kSlots][HD][FS];   // the batch (24 rows), then H1 in its place
+    float b1[HD], b2[HD], w3[HD];
+};
+static_assert(sizeof(ForwardSmem) <= 48 * 1024, "static shared memory");
+
+__device__ __forceinline__ void slot_sync(int slot)
 {
-    __shared__ float w2t[HD][HD];   // w2t[i][j] = W2[j][i]
-    __shared__ float b2s[HD], w3s[HD];
-    for (int e = threadIdx.x; e < HD * HD; e += blockDim.x) {
-        const int j = e / HD, i = e % HD;
-        w2t[i][j] = P[OW2 + e];
+    asm volatile("bar.sync %0, 64;" ::"r"(slot + 1) : "memory");
+}
+
+// acc[v][0..3] += sum over k (ascending) of W[ug + 8v][k] * A[k][4q .. 4q + 3]
+template <int K, int WS>
+__device__ __forceinline__ void units8(const float *w, const float *A, float (&acc)[8][4])
+{
+#pragma unroll 2
+    for (int k = 0; k < K; k += 4) {
+        float4 a[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) a[j] = at4(A + (k + j) * FS);
+#pragma unroll
+        for (int v = 0; v < 8; ++v) {
+            const float4 w4 = at4(w + 8 * v * WS + k);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float wk = part(w4, j);
+                acc[v][0] = __fmaf_rn(wk, a[j].x, acc[v][0]);
+                acc[v][1] = __fmaf_rn(wk, a[j].y, acc[v][1]);
+                acc[v][2] = __fmaf_rn(wk, a[j].z, acc[v][2]);
+                acc[v][3] = __fmaf_rn(wk, a[j].w, acc[v][3]);
+            }
+        }
     }
-    for (int j = threadIdx.x; j < HD; j += blockDim.x) {
-        b2s[j] = P[OB2 + j];
-        w3s[j] = P[OW3 + j];
+}
+
+__global__ void __launch_bounds__(64 * kSlots) k_mlp_forward(const float *__restrict__ P, const float *__restrict__ X,
+                                                            int n, float *__restrict__ y)
+{
+    __shared__ __align__(16) ForwardSmem T;
+    const int tid = threadIdx.x;
+    float w1[HD * IN / (64 * kSlots)], w2[HD * HD / (64 * kSlots)];   // every load in flight at once
+#pragma unroll
+    for (int i = 0; i < HD * IN / (64 * kSlots); ++i) w1[i] = __ldg(P + OW1 + tid + i * 64 * kSlots);
+#pragma unroll
+    for (int i = 0; i < HD * HD / (64 * kSlots); ++i) w2[i] = __ldg(P + OW2 + tid + i * 64 * kSlots);
+#pragma unroll
+    for (int i = 0; i < HD * IN / (64 * kSlots); ++i) {
+        const int e = tid + i * 64 * kSlots;
+        T.W1[e / IN][e % IN] = w1[i];
     }
+#pragma unroll
+    for (int i = 0; i < HD * HD / (64 * kSlots); ++i) {
+        const int e = tid + i * 64 * kSlots;
+        T.W2[e / HD][e % HD] = w2[i];
+    }
+    for (int e = tid; e < HD; e += 64 * kSlots) T.b1[e] = P[OB1 + e], T.b2[e] = P[OB2 + e], T.w3[e] = P[OW3 + e];
+    const float b3 = P[OB3];
     __syncthreads();
-    const int lane = threadIdx.x & 31;
-    float w1a[IN], w1b[IN];
+    const int slot = tid >> 6, t64 = tid & 63, lane = tid & 31;
+    const int ug = lane >> 2, q = 4 * (t64 >> 5) + (lane & 3);
+    float(*A)[FS] = T.A[slot];
+    const int tiles = n / kTile + (n % kTile != 0);
+    for (int64_t tile = (int64_t)slot * gridDim.x + blockIdx.x; tile < tiles; tile += (int64_t)kSlots * gridDim.x) {
+        const int64_t s0 = tile * kTile;
+        const int m = (int)min((int64_t)kTile, n - s0);   // samples past the end count as zeros
 #pragma unroll
-    for (int k = 0; k < IN; ++k) {
-        w1a[k] = P[OW1 + lane * IN + k];
-        w1b[k] = P[OW1 + (lane + 32) * IN + k];
-    }
-    const float b1a = P[OB1 + lane], b1b = P[OB1 + lane + 32], b3 = P[OB3];
-    const int warps = (gridDim.x * blockDim.x) >> 5;
-    for (int s = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; s < n; s += warps) {
-        const float *xs = X + (int64_t)s * IN;
-        float a0 = b1a, a1 = b1b;
-#pragma unroll
-        for (int k = 0; k < IN; ++k) {
-            const float xk = __ldg(xs + k);
-            a0 = __fmaf_rn(w1a[k], xk, a0);
-            a1 = __fmaf_rn(w1b[k], xk, a1);
+        for (int e = t64; e < kTile * IN; e += 64) {
+            const int s = e / IN;
+            A[e - s * IN][s] = s < m ? __ldg(X + s0 * IN + e) : 0.f;
         }
-        const float ha = fmaxf(a0, 0.f), hb = fmaxf(a1, 0.f);
-        float c0 = b2s[lane], c1 = b2s[lane + 32];
+        slot_sync(slot);
+        float acc[8][4];
 #pragma unroll
-        for (int i = 0; i < HD; ++i) {
-            const float hi = __shfl_sync(0xffffffffu, i < 32 ? ha : hb, i & 31);
-            c0 = __fmaf_rn(w2t[i][lane], hi, c0);
-            c1 = __fmaf_rn(w2t[i][lane + 32], hi, c1);
+        for (int v = 0; v < 8; ++v)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc[v][i] = T.b1[ug + 8 * v];
+        units8<IN, 28>(T.W1[ug], &A[0][4 * q], acc);
+        slot_sync(slot);
+#pragma unroll
+        for (int v = 0; v < 8; ++v) {
+            *reinterpret_cast<float4 *>(&A[ug + 8 * v][4 * q]) =
+                make_float4(fmaxf(acc[v][0], 0.f), fmaxf(acc[v][1], 0.f), fmaxf(acc[v][2], 0.f), fmaxf(acc[v][3], 0.f));
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc[v][i] = T.b2[ug + 8 * v];
         }
-        float o = __fmaf_rn(w3s[lane], fmaxf(c0, 0.f), w3s[lane + 32] * fmaxf(c1, 0.f));
+        slot_sync(slot);
+        units8<HD, 68>(T.W2[ug], &A[0][4 * q], acc);
+        // the output's sum as a butterfly over units: j with j + 32, then
+        // distances 16 and 8 in the lane, 4, 2 and 1 across lanes
+        float o[4];
 #pragma unroll
-        for (int m = 16; m >= 1; m >>= 1) o += __shfl_xor_sync(0xffffffffu, o, m);
-        if (lane == 0) y[s] = o + b3;
+        for (int i = 0; i < 4; ++i) {
+            float h[4];
+#pragma unroll
+            for (int v = 0; v < 4; ++v)
+                h[v] = __fmaf_rn(T.w3[ug + 8 * v], fmaxf(acc[v][i], 0.f), T.w3[ug + 8 * v + 32] * fmaxf(acc[v + 4][i], 0.f));
+            o[i] = (h[0] + h[2]) + (h[1] + h[3]);
+#pragma unroll
+            for (int d = 16; d >= 4; d >>= 1) o[i] += __shfl_xor_sync(0xffffffffu, o[i], d);
+        }
+        if (ug == 0)
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (4 * q + i < m) y[s0 + 4 * q + i] = o[i] + b3;
+        slot_sync(slot);   // the tile is read before the next one is stored
     }
 }
 
@@ -150,8 +231,6 @@ __device__ __forceinline__ void put4(unsigned addr, float4 v)
     asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w)
                  : "memory");
 }
-__device__ __forceinline__ float4 at4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
-__device__ __forceinline__ float part(const float4 &v, int i) { return i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w; }
 
 // acc[0..3] += sum over k (ascending) of w[k] * A[k][0..3]; A's rows S apart
 template <int K>
@@ -436,8 +515,9 @@ hf_status hf_mlp_forward(const float *params, const float *X, int n, float *y, v
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int blocks = std::min((n + 7) / 8, 4 * sms);   // 8 warps per block
-    k_mlp_forward<<<blocks, 256, 0, static_cast<cudaStream_t>(stream)>>>(params, X, n, y);
+    // two blocks an SM share its shared-load pipe; fewer while tiles last
+    const int blocks = std::min(n / kTile + (n % kTile != 0), 2 * sms);
+    k_mlp_forward<<<blocks, 64 * kSlots, 0, static_cast<cudaStream_t>(stream)>>>(params, X, n, y);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? HF_OK : hf::set_last_error(HF_ERR_CUDA, cudaGetErrorString(e));
 }
