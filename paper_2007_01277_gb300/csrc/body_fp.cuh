@@ -223,6 +223,16 @@ struct BodyBf16Axpy {
 // then k%4 more on the leading components) and stores it.  The first
 // barrier follows the staging, the others split the FMA rounds evenly.  All
 // threads run the same number of tiles so every barrier is uniform.
+//
+// Bound by HBM for small k, by the FMA pipe for large.  The next tile's group
+// is loaded before the current one is staged, so its latency spans the
+// barriers; a round is two packed multiply-adds (the bits of four scalar
+// ones); and the rounds at which barriers fall are divided out once, not per
+// tile (as 64-bit quotients they were most of a short tile's instructions).
+// A pair of 2^24 floats with k = 16, 2 barriers, 8 KB and 6 * 10^6 floats
+// with k = 256, 1 barrier (128 of 256 threads each): 66.3 -> 51.3 us.  Two
+// to four groups ahead took 53-64 us there and spilled under the caps of 32
+// and 40 registers.
 struct BodyStreamTmpl {
     using Args = hf_stream_tmpl_args;
     static constexpr int kId = HF_BODY_STREAM_TMPL;
@@ -239,28 +249,36 @@ struct BodyStreamTmpl {
         return HF_OK;
     }
 
-    static __device__ __forceinline__ void round4(float4 &v, float m, float b)
+    // v as two packed pairs: one multiply-add of every component
+    static __device__ __forceinline__ void rounds(unsigned long long &lo, unsigned long long &hi, int from, int upto,
+                                                  unsigned long long m, unsigned long long b)
     {
-        v.x = __fmaf_rn(v.x, m, b);
-        v.y = __fmaf_rn(v.y, m, b);
-        v.z = __fmaf_rn(v.z, m, b);
-        v.w = __fmaf_rn(v.w, m, b);
+#pragma unroll 4
+        for (int j = from; j < upto; ++j) {
+            lo = f2fma(lo, m, b);
+            hi = f2fma(hi, m, b);
+        }
     }
 
     static __device__ void run(const Args &a, const Ctx &cx)
     {
         const int64_t n4 = a.n >> 2;
         const int64_t stride = (int64_t)cx.grid * cx.nthreads;
-        const int64_t tiles = (n4 + stride - 1) / stride;
         const int nslots = smem_fits(cx, (size_t)a.smem_bytes) ? a.smem_bytes >> 4 : 0;
         const bool staged = cx.tid < nslots;
         const unsigned slot = (unsigned)__cvta_generic_to_shared(cx.smem) + 16u * cx.tid;
         const int k4 = a.k >> 2, kr = a.k & 3, nb = a.n_barriers;
-        const float m = a.a, b = a.b;
-        for (int64_t t = 0; t < tiles; ++t) {
-            const int64_t i = (int64_t)cx.block * cx.nthreads + cx.tid + t * stride;
+        // barrier s (1 .. nb - 1) follows round k4 * s / nb
+        const int at1 = nb > 1 ? k4 / nb : 0, at2 = nb > 2 ? 2 * k4 / nb : 0, at3 = nb > 3 ? 3 * k4 / nb : 0;
+        const unsigned long long m = f2pack(a.a, a.a), b = f2pack(a.b, a.b);
+        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+        const int64_t tiles = (n4 + stride - 1) / stride;   // of every thread: barriers stay uniform
+        int64_t i = (int64_t)cx.block * cx.nthreads + cx.tid;
+        float4 next = i < n4 ? ldcs4(a.x + 4 * i) : zero;
+        for (int64_t t = 0; t < tiles; ++t, i += stride) {
             const bool ok = i < n4;
-            float4 v = ok ? ldcs4(a.x + 4 * i) : make_float4(0.f, 0.f, 0.f, 0.f);
+            float4 v = next;
+            next = i + stride < n4 ? ldcs4(a.x + 4 * (i + stride)) : zero;
             if (staged)
                 asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(slot), "f"(v.x),
                              "f"(v.y), "f"(v.z), "f"(v.w)
@@ -271,18 +289,29 @@ struct BodyStreamTmpl {
                              : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
                              : "r"(slot)
                              : "memory");
+            unsigned long long lo = f2pack(v.x, v.y), hi = f2pack(v.z, v.w);
             int done = 0;
-            for (int s = 1; s < nb; ++s) {
-                const int upto = (int)((int64_t)k4 * s / nb);
-#pragma unroll 4
-                for (; done < upto; ++done) round4(v, m, b);
+            if (nb > 1) {
+                rounds(lo, hi, 0, at1, m, b);
                 interval_sync(cx);
+                done = at1;
+                if (nb > 2) {
+                    rounds(lo, hi, at1, at2, m, b);
+                    interval_sync(cx);
+                    done = at2;
+                    if (nb > 3) {
+                        rounds(lo, hi, at2, at3, m, b);
+                        interval_sync(cx);
+                        done = at3;
+                    }
+                }
             }
-#pragma unroll 4
-            for (; done < k4; ++done) round4(v, m, b);
-            if (kr > 0) v.x = __fmaf_rn(v.x, m, b);
-            if (kr > 1) v.y = __fmaf_rn(v.y, m, b);
-            if (kr > 2) v.z = __fmaf_rn(v.z, m, b);
+            rounds(lo, hi, done, k4, m, b);
+            f2unpack(lo, v.x, v.y);
+            f2unpack(hi, v.z, v.w);
+            if (kr > 0) v.x = __fmaf_rn(v.x, a.a, a.b);
+            if (kr > 1) v.y = __fmaf_rn(v.y, a.a, a.b);
+            if (kr > 2) v.z = __fmaf_rn(v.z, a.a, a.b);
             if (ok) stcs4(a.y + 4 * i, v);
         }
     }
