@@ -14,6 +14,7 @@
 //              bodies, optionally bounded by __maxnreg__ (Algorithm 2's r0)
 #pragma once
 #include <cstring>
+#include <type_traits>
 
 #include "hf_launch.h"
 
@@ -64,6 +65,26 @@ template <class B>
 __global__ void k_single(const __grid_constant__ SingleParams<B> p)
 {
     single_body<B>(p);
+}
+
+// The same with the registers that blocks of 1024 threads leave, for bodies
+// that declare kFullBlock: launches that k_single's registers do not allow.
+template <class B>
+__global__ void __launch_bounds__(1024) k_single_full(const __grid_constant__ SingleParams<B> p)
+{
+    single_body<B>(p);
+}
+template <class B, class = void>
+struct FullBlock : std::false_type {
+};
+template <class B>
+struct FullBlock<B, std::void_t<decltype(B::kFullBlock)>> : std::true_type {
+};
+template <class B>
+const void *single_full_func()
+{
+    if constexpr (FullBlock<B>::value) return reinterpret_cast<const void *>(&k_single_full<B>);
+    return nullptr;
 }
 
 // ------------------------------------------------------------------ pair
@@ -252,13 +273,24 @@ unsigned *error_word();
 using hfl::Instance;     // registry entry of one compiled instance
 using hfl::PairLaunch;   // arguments of one 2-way launch
 
+// The bound an instance of cap R is compiled with: R, or a lower one where
+// the compiler would spend registers below R that cost larger blocks and
+// give nothing.
+template <class A, class B>
+constexpr int compiled_cap(int r)
+{
+    // 94 registers below a cap of 96 would end blocks of 768 threads
+    if (A::kId == HF_BODY_SHA256D && B::kId == HF_BODY_BLAKE2B && r == 96) return 80;
+    return r;
+}
+
 template <class A, class B, int R>
 const void *pair_func()
 {
     if constexpr (R == 0)
         return reinterpret_cast<const void *>(&k_pair<A, B>);
     else
-        return reinterpret_cast<const void *>(&k_pair_cap<A, B, R>);
+        return reinterpret_cast<const void *>(&k_pair_cap<A, B, compiled_cap<A, B>(R)>);
 }
 
 template <class A, class B, int R>
@@ -299,13 +331,14 @@ const Instance *nway_table(int *n);
 // Standalone kernels: one per body, no register bound.
 struct SingleEntry {
     int body;
-    const void *func;
-    cudaError_t (*launch)(const void *args, int threads, int grid, unsigned smem, unsigned *err,
+    const void *func;        // k_single
+    const void *func_full;   // k_single_full, or nullptr
+    cudaError_t (*launch)(const void *func, const void *args, int threads, int grid, unsigned smem, unsigned *err,
                           unsigned ring_stage, int ring_stages, cudaStream_t);
 };
 
 template <class B>
-cudaError_t launch_single(const void *args, int threads, int grid, unsigned smem, unsigned *err,
+cudaError_t launch_single(const void *func, const void *args, int threads, int grid, unsigned smem, unsigned *err,
                           unsigned ring_stage, int ring_stages, cudaStream_t s)
 {
     SingleParams<B> p;
@@ -315,8 +348,7 @@ cudaError_t launch_single(const void *args, int threads, int grid, unsigned smem
     p.ring_stage = ring_stage;
     p.ring_stages = ring_stages;
     void *kargs[] = {&p};
-    return cudaLaunchKernel(reinterpret_cast<const void *>(&k_single<B>), dim3(grid),
-                            dim3(threads), kargs, smem, s);
+    return cudaLaunchKernel(func, dim3(grid), dim3(threads), kargs, smem, s);
 }
 
 const SingleEntry *single_table(int *n);

@@ -478,13 +478,23 @@ void interval_smem_at(const int *ids, const void *const *args, const int *thread
 } // namespace hf
 
 namespace {
-hf_status single_plan(const hf_kernel_t *k, const void *args, int threads, int want, LaunchPlan *plan)
+// The kernel of a body launched alone on blocks of `threads`, and its info.
+hf_status single_kernel(const SingleEntry *e, int threads, const void **func, FuncInfo *fi)
 {
-    const SingleEntry *e = find_single(k->body);
+    *func = e->func;
+    hf_status s = func_info(e->func, fi);
+    if (s || fi->max_threads >= threads || !e->func_full) return s;
+    *func = e->func_full;
+    return func_info(e->func_full, fi);
+}
+
+hf_status single_plan(const hf_kernel_t *k, const void *func, const void *args, int threads, int want,
+                      LaunchPlan *plan)
+{
     const size_t base = body_ops(k->body).smem(threads, args);
     const int ring = body_ops(k->body).ring(args);
     const unsigned ring_min = body_ops(k->body).ring_min;
-    return plan_launch(e->func, threads, 1, &threads, &base, &ring, &ring_min, want, plan);
+    return plan_launch(func, threads, 1, &threads, &base, &ring, &ring_min, want, plan);
 }
 
 hf_status validate_args(int body, const void *a, int which)
@@ -879,14 +889,15 @@ hf_status hf_launch_single(hf_kernel k, const void *args, int threads, int grid,
     if (s) return s;
     const SingleEntry *e = find_single(k->body);
     FuncInfo fi;
-    s = func_info(e->func, &fi);
+    const void *func;
+    s = single_kernel(e, threads, &func, &fi);
     if (s) return s;
     if (fi.max_threads < threads)
         return fail(HF_ERR_REGS, "kernel uses %d registers: at most %d threads", fi.regs, fi.max_threads);
     LaunchPlan plan;
-    s = single_plan(k, args, threads, grid, &plan);
+    s = single_plan(k, func, args, threads, grid, &plan);
     if (s) return s;
-    HF_CUDA(e->launch(args, threads, plan.grid, plan.smem, hf::error_word(), plan.ring_stage[0],
+    HF_CUDA(e->launch(func, args, threads, plan.grid, plan.smem, hf::error_word(), plan.ring_stage[0],
                       plan.ring_stages[0], static_cast<cudaStream_t>(stream)));
     return HF_OK;
 }
@@ -926,10 +937,11 @@ hf_status hf_query_single(hf_kernel k, const void *args, int threads, hf_fused_i
     if (s) return s;
     const SingleEntry *e = find_single(k->body);
     FuncInfo fi;
-    s = func_info(e->func, &fi);
+    const void *func;
+    s = single_kernel(e, threads, &func, &fi);
     if (s) return s;
     LaunchPlan plan;
-    s = single_plan(k, args, threads, 0, &plan);
+    s = single_plan(k, func, args, threads, 0, &plan);
     if (s) return s;
     const size_t smem = plan.smem;
     const int bps = plan.bps;
