@@ -800,33 +800,30 @@ struct BodyMaxpool {
 };
 
 // ------------------------------------------------------------------------
-// im2col, 3x3 window, stride 1, padding 1.  Vector path (W % 4 == 0,
-// W <= 64): a warp takes a chunk of rows of one (n, c) plane, each half-warp
+// im2col, 3x3 window, stride 1, padding 1: the flat path where three rows fit
+// a ring's stage (or strips, below).  Without a ring, the vector path (W % 4
+// == 0, W <= 64): a warp takes a chunk of rows of one (n, c) plane, each half-warp
 // half of the chunk; lane holds 4 columns of three consecutive input rows
 // and writes the nine shifted copies (ky, kx) of its columns for each row.
 struct BodyIm2col {
     using Args = hf_im2col3_args;
     static constexpr int kId = HF_BODY_IM2COL3;
     static constexpr int kBarriers = 0;
-    // ring path: a stage holds an item's 14 rows and its two halo rows
-    // (rows of up to 64 floats), or at least three rows (the flat path)
-    static constexpr int kRingRows = 14;
+    // ring path: a stage holds at least three rows (the flat path).  Strips
+    // of whole 16-byte rows, a half-warp a row, take fewer instructions: at W =
+    // 56 and 64 a lone warp an SM took 93 and 89 us for 2^23 values, flat 101
+    // and 108 -- level from two warps on, and strips 1.2 to 4.7 times slower
+    // at W = 48 .. 16.  So they are kept for a lone warp's interval of an
+    // N-way schedule (the 8-way launch 392.9 us, 395.4 without) and compiled
+    // there only: beside the flat path they cost pairs capped at 64 registers
+    // 100 bytes of spills and 5 to 11 % (histogram + im2col).
+    static constexpr int kRingRows = 14;   // rows of a strip item
+    static constexpr int kStripCols = 56;
     static constexpr bool kRingItem = true;
     static constexpr unsigned kRingMinBytes = 4096;   // the stage: one item
-    // Strips of 16-byte rows of 56 to 64 values, the flat path for all others.
-    // Both are at the write rate from four warps an SM on; with one warp an
-    // SM (an interval of a large schedule), where instructions count, 2^23
-    // values of W = 16 / 28 / 48 / 56 / 64 columns took strips 493 / 171 /
-    // 121 / 93 / 89 us and the flat path 105 / 105 / 109 / 101 / 108.
-    static constexpr int kStripCols = 56;
-    static __host__ __device__ bool rows16(const Args &a)
-    {
-        return (a.W & 3) == 0 && a.W <= 64 && aligned16(a.x) && aligned16(a.col);
-    }
     static __host__ bool uses_ring(const Args &a)
     {
-        if ((int64_t)a.N * a.C * a.H * a.W <= 0) return false;
-        return (rows16(a) && a.W >= kStripCols) || (aligned16(a.x) && 3u * a.W + kFlatPad <= kRingMinBytes / 4);
+        return (int64_t)a.N * a.C * a.H * a.W > 0 && aligned16(a.x) && 3u * a.W + kFlatPad <= kRingMinBytes / 4;
     }
 
     static __host__ size_t workspace_bytes(const Args &) { return 0; }
@@ -1150,21 +1147,26 @@ struct BodyIm2col {
         }
     }
 
-    static __device__ void run(const Args &a, const Ctx &cx)
+    // STRIPS: with the strip path for a lone warp's interval (N-way schedules)
+    template <bool STRIPS>
+    static __device__ __forceinline__ void run_as(const Args &a, const Ctx &cx)
     {
         if ((int64_t)a.N * a.C * a.H * a.W == 0) return;
         const bool flat = flat_range((int64_t)a.N * a.C * a.H, a.W, cx);
-        if (rows16(a) && a.W >= kStripCols) {
-            if (WarpRing::available(cx, 0) && run_ring(a, cx)) return;
-        } else if (flat) {
+        if (STRIPS && cx.nthreads == 32 && (a.W & 3) == 0 && a.W >= kStripCols && a.W <= 64 && aligned16(a.x) &&
+            aligned16(a.col) && WarpRing::available(cx, 0) && run_ring(a, cx))
+            return;
+        if (flat) {
             const bool v4 = a.W >= 4 && ((int64_t)a.H * a.W & 3) == 0 && aligned16(a.col);
             if (v4 && flat_ring<4>(a, cx)) return;
             if (flat_ring<1>(a, cx)) return;
         }
-        if (rows16(a)) run_vec(a, cx);
+        if ((a.W & 3) == 0 && a.W <= 64 && aligned16(a.x) && aligned16(a.col)) run_vec(a, cx);
         else if (flat) flat_global(a, cx);
         else run_scalar(a, cx);
     }
+
+    static __device__ void run(const Args &a, const Ctx &cx) { run_as<false>(a, cx); }
 };
 
 } // namespace hf

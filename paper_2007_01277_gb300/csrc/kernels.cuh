@@ -192,7 +192,7 @@ __device__ __forceinline__ void dispatch(const NwayParams &p, int j, const Ctx &
         BodyMaxpool::run(*reinterpret_cast<const BodyMaxpool::Args *>(args), c);
         break;
     case HF_BODY_IM2COL3:
-        BodyIm2col::run(*reinterpret_cast<const BodyIm2col::Args *>(args), c);
+        BodyIm2col::run_as<true>(*reinterpret_cast<const BodyIm2col::Args *>(args), c);
         break;
     case HF_BODY_HIST256: BodyHist::run(*reinterpret_cast<const BodyHist::Args *>(args), c); break;
     case HF_BODY_PHILOX:
