@@ -243,11 +243,26 @@ def _check(fn, status):
         raise HFError(fn, status, lib.hf_last_error().decode())
 
 
+_raw_stream = None
+
+
+def _current_stream():
+    """The current stream's handle.  Once CUDA is up, without the Stream
+    object that torch.cuda.current_stream() builds on every call."""
+    global _raw_stream
+    if _raw_stream is None:
+        import torch
+        ptr = torch.cuda.current_stream().cuda_stream   # initialises CUDA
+        get, dev = (getattr(torch._C, n, None) for n in ("_cuda_getCurrentRawStream", "_cuda_getDevice"))
+        _raw_stream = (lambda: get(dev())) if get and dev else (lambda: torch.cuda.current_stream().cuda_stream)
+        return ptr
+    return _raw_stream()
+
+
 def _stream_ptr(stream):
     """A torch.cuda.Stream, a raw cudaStream_t int, or None (current stream)."""
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        return _current_stream()
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
@@ -285,17 +300,26 @@ def hf_fuse_n(kernels, interval_of, interval_threads, regcap=0):
     return h
 
 
+_addr = ctypes.addressof
+_ARGV = [_P * n for n in range(MAX_SCHEDULE + 1)]
+
+
 def _argv(args):
-    return (_P * len(args))(*[ctypes.cast(ctypes.pointer(a), _P) for a in args])
+    # the blocks' addresses: they are read before the call returns
+    n = len(args)
+    return (_ARGV[n] if n <= MAX_SCHEDULE else _P * n)(*[_addr(a) for a in args])
 
 
 def hf_launch(f, args, grid=0, stream=None):
-    _check("hf_launch", lib.hf_launch(f, _argv(args), grid, _stream_ptr(stream)))
+    s = lib.hf_launch(f, _argv(args), grid, _stream_ptr(stream))
+    if s:
+        _check("hf_launch", s)
 
 
 def hf_launch_single(k, args, threads, grid=0, stream=None):
-    _check("hf_launch_single", lib.hf_launch_single(k, ctypes.cast(ctypes.pointer(args), _P),
-                                                    threads, grid, _stream_ptr(stream)))
+    s = lib.hf_launch_single(k, _addr(args), threads, grid, _stream_ptr(stream))
+    if s:
+        _check("hf_launch_single", s)
 
 
 def hf_query(f, args):
