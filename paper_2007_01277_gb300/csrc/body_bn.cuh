@@ -8,7 +8,8 @@
 // of tiles through a counter in shared memory).  A tile arrives either
 // through the warp's bulk-copy ring (its one to three runs copied into one
 // stage, the next tiles' copies in flight) or, without a ring, as 128-bit
-// loads, 16 per lane with 8 in flight.  Each tile yields FP32 sums of
+// loads, 16 per lane with 8 in flight (32-bit loads, 64 with 16 in flight,
+// where HW or the alignment needs them).  Each tile yields FP32 sums of
 // d = x - K_c and d*d, where the shift K_c = x[0][c][0] keeps the variance
 // free of cancellation (the shifted-data algorithm, Chan, Golub & LeVeque
 // 1983), in the same order on both paths.  A warp writes the tile's pair to
@@ -73,7 +74,7 @@ struct BodyBn {
     // The tile's FP32 sums of d = x - K and d*d, in the one order every
     // path uses: lane l takes the VEC values at tile offsets VEC*l + 32*VEC*k
     // for k = 0, 1, ... (values past the channel's end read as K, so d = 0),
-    // in batches of 8 steps whose values get(k) returns -- the batch's
+    // in batches of kBatch steps whose values get(k) returns -- the batch's
     // loads are all issued before its arithmetic; four per-lane sums (two
     // packed pairs for VEC = 4), then their sum and a warp butterfly.
     template <int VEC, class Get>
@@ -87,7 +88,12 @@ struct BodyBn {
         unsigned long long P1a = f2pack(0.f, 0.f), P1b = P1a, P2a = P1a, P2b = P1a;
         const unsigned long long KK = f2pack(K, K);
         constexpr int kSteps = kTile / (32 * VEC);
-        constexpr int kBatch = 8;
+        // Loads in flight per lane.  Single values need more of them: 16
+        // against 8 took 64x64x75x75 from 35.3 to 22.3 us and 64x512x7x7 from
+        // 11.4 to 9.1 (with the pointer kept below instead of a product per
+        // value); 32 gave another 1 to 3 %, but registers that end blocks of
+        // 768 threads of batch-norm + polynomial capped at 96.
+        constexpr int kBatch = VEC == 4 ? 8 : 16;
 #pragma unroll 1
         for (int s = 0; s < kSteps; s += kBatch) {
             float vals[kBatch][VEC];
@@ -146,12 +152,14 @@ struct BodyBn {
         // (n, hw) of this lane's first value; later values advance by 32*VEC.
         int n = (int)(j0 / a.HW);
         int hw = (int)(j0 - (int64_t)n * a.HW);
+        // values of this lane's steps that the channel has: j0 + 32*VEC*k < jend
         const int64_t jend = (t + 1) * kTile < M ? (t + 1) * kTile : M;
-        int64_t j = j0;
+        int left = (int)(jend - j0);
+        const float *p = a.x + ((int64_t)n * a.C + c) * a.HW + hw;
+        const int64_t skip = (int64_t)(a.C - 1) * a.HW;   // from a run's end to the channel's next run
         accumulate<VEC>(
             [&](int, float(&v)[VEC]) {
-                const bool ok = j < jend;
-                const float *p = a.x + ((int64_t)n * a.C + c) * a.HW + hw;
+                const bool ok = left > 0;
                 if (VEC == 4) {
                     const float4 q = ok ? ldcs4(p) : make_float4(K, K, K, K);
                     v[0] = q.x;
@@ -161,11 +169,12 @@ struct BodyBn {
                 } else {
                     v[0] = ok ? __ldcs(p) : K;
                 }
-                j += 32 * VEC;
+                left -= 32 * VEC;
+                p += 32 * VEC;
                 hw += 32 * VEC;
                 while (hw >= a.HW) {
                     hw -= a.HW;
-                    ++n;
+                    p += skip;
                 }
             },
             K, s1, s2);

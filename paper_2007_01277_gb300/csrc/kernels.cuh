@@ -287,6 +287,12 @@ constexpr int compiled_cap(int r)
 template <class A, class B, int R>
 const void *pair_func()
 {
+#ifdef HF_CHECKED_BARRIERS
+    // 76 registers otherwise, where blocks of 896 threads need 72
+    if constexpr (R == 0 && A::kId == HF_BODY_BN_STATS && B::kId == HF_BODY_HIST256)
+        return reinterpret_cast<const void *>(&k_pair_cap<A, B, 72>);
+    else
+#endif
     if constexpr (R == 0)
         return reinterpret_cast<const void *>(&k_pair<A, B>);
     else
