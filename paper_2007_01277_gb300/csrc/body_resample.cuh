@@ -43,12 +43,14 @@ struct ItemCursor {
 // from global memory.  Only the division of a pixel's index by the row
 // length remains, a multiply and a shift (indices stay below 1024).
 //
-// The bound is HBM; one 32-pixel step of upsample moves 640 bytes in about
-// 45 issue slots, where an SM has about 108 for them.  It replaces paths of
+// The bound is HBM at full occupancy and issue in a fused block of few warps:
+// 32 pixels of upsample move 640 bytes, for which an SM has about 108 issue
+// slots, and take about 100.  It replaces paths of
 // one thread per output with two 64-bit divisions each.  On one GB300, before
-// -> with it: upsample 8x64x75x75 + max pool 8x64x147x147 fused 287 -> 27.7
-// us, im2col 8x64x112x112 alone 309 -> 46.2 us (5.6 TB/s), batch-norm
-// 64x512x7x7 + im2col 32x256x14x14 fused 243 -> 22.3 us.
+// -> with it: upsample 8x64x75x75 + max pool 8x64x147x147 fused 287 -> 28.2
+// us, im2col 8x64x112x112 alone 309 -> 46.0 us (5.6 TB/s), batch-norm
+// 64x512x7x7 + im2col 32x256x14x14 fused 243 -> 22.3 us (18.6 with the
+// statistics' deeper loads).
 struct FlatRows {
     unsigned W, H, R;    // values per row, rows per plane, rows per item
     unsigned rows;       // rows of all planes

@@ -176,11 +176,12 @@ __global__ void __launch_bounds__(64 * kSlots) k_mlp_forward(const float *__rest
 // finished the step before.  Two warps gather the next step's batch meanwhile.
 //
 // The bound is latency: a step is a chain of five products of 24 to 64
-// dependent multiply-adds, two cluster barriers and five block barriers, and
-// about 1000 cycles of multiply-add issue per block.  A single block with
+// dependent multiply-adds, five block barriers and two exchanges of 16 KB
+// over distributed shared memory, about 3500 of its 17000 cycles each (bulk
+// copies and asynchronous stores with mbarriers took as long).  A single block with
 // one output per thread and both operands from shared memory (10 block
 // barriers, its load pipe 65 % busy) took 37.3 us a step at batch 64;
-// this takes 8.1 us, with the same bits.  Every sum keeps one fixed order (inputs or samples
+// this takes 8.2 us, with the same bits.  Every sum keeps one fixed order (inputs or samples
 // ascending), so a run is deterministic; samples past the batch count as zero.
 constexpr int kCl = 8, kU = HD / kCl;    // blocks of the cluster, units per block
 constexpr int kWarps = 11, kTrainThreads = 32 * kWarps;
