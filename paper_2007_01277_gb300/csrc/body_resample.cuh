@@ -47,7 +47,7 @@ struct ItemCursor {
 // 32 pixels of upsample move 640 bytes, for which an SM has about 108 issue
 // slots, and take about 100.  It replaces paths of
 // one thread per output with two 64-bit divisions each.  On one GB300, before
-// -> with it: upsample 8x64x75x75 + max pool 8x64x147x147 fused 287 -> 28.2
+// -> with it: upsample 8x64x75x75 + max pool 8x64x147x147 fused 287 -> 26.6
 // us, im2col 8x64x112x112 alone 309 -> 46.0 us (5.6 TB/s), batch-norm
 // 64x512x7x7 + im2col 32x256x14x14 fused 243 -> 22.3 us (18.6 with the
 // statistics' deeper loads).
@@ -77,6 +77,29 @@ struct FlatRows {
     // row t of that plane's run of rows, t < H + R
     __device__ unsigned row_of(unsigned i) const { return R == 1 ? 0u : (i * mw) >> 20; }
     __device__ unsigned plane_of(unsigned t) const { return H <= 1024 ? (t * mh) >> 21 : (t >= H ? 1u : 0u); }
+};
+
+// Plane p and row r in it of the first row of a warp's items it, it + step,
+// ..., advanced without divisions: in items of few pixels, as max pool's two
+// rows of 74, those were a fifth of the instructions (upsample 8x64x75x75 +
+// max pool 8x64x147x147 28.4 -> 26.6 us; im2col, bound by its stores, gained
+// nothing and divides).
+struct FlatCursor {
+    unsigned p, r, dp, dr;
+    __device__ void init(const FlatRows &f, int64_t it, int64_t step)
+    {
+        const uint64_t row = it < (int64_t)f.items() ? (uint64_t)it * f.R : 0, d = (uint64_t)step * f.R;
+        p = (unsigned)(row / f.H);
+        r = (unsigned)(row - (uint64_t)p * f.H);
+        dp = (unsigned)(d / f.H);   // beyond 32 bits only where no second item exists
+        dr = (unsigned)(d - d / f.H * f.H);
+    }
+    __device__ void step(unsigned H)
+    {
+        p += dp;
+        r += dr;
+        if (r >= H) r -= H, ++p;
+    }
 };
 
 // Reads of an item's values at offsets from its first pixel: from the stage,
@@ -367,11 +390,10 @@ struct BodyUpsample {
     // One item of the flat path: pixel i gives the outputs (2r, 2r+1) x
     // (2c, 2c+1); in memory they start at 4*i - 2*c from the item's first.
     template <class Get>
-    static __device__ __forceinline__ void flat_item(const Args &a, const FlatRows &f, unsigned g0, unsigned n,
-                                                     const Get &get)
+    static __device__ __forceinline__ void flat_item(const Args &a, const FlatRows &f, unsigned g0, unsigned r0,
+                                                     unsigned n, const Get &get)
     {
         const int W = (int)f.W;
-        const unsigned r0 = g0 % f.H;
         float *y0 = a.y + 4 * (int64_t)g0 * W;
         const bool y8 = (reinterpret_cast<uintptr_t>(a.y) & 7u) == 0;
 #pragma unroll 2
@@ -414,6 +436,8 @@ struct BodyUpsample {
         f.init(W, a.H, (unsigned)rows, min((slots - kFlatPad) / W - 2, FlatRows::kMaxValues / W), (unsigned)GW, 1);
         WarpRing r;
         r.init(cx, 0);
+        FlatCursor uc;
+        uc.init(f, gw, GW);
         auto copy = [&](int64_t it) {
             const int64_t g0 = it * f.R;
             return FlatCopy((g0 - 1) * W - 1, (min(g0 + (int64_t)f.R, rows) + 1) * W + 1, total);
@@ -424,8 +448,9 @@ struct BodyUpsample {
                 const int64_t g0 = it * f.R, g1 = min(g0 + (int64_t)f.R, rows);
                 const FlatCopy k = copy(it);
                 k.patch(stage, a.x, (g1 + 1) * W + 1, total, r.lane);
-                flat_item(a, f, (unsigned)g0, (unsigned)(g1 - g0) * W,
+                flat_item(a, f, (unsigned)g0, uc.r, (unsigned)(g1 - g0) * W,
                           FlatStage{reinterpret_cast<const float *>(stage) + (g0 * W - k.base)});
+                uc.step(f.H);
             });
         r.finish();
         return true;
@@ -442,7 +467,7 @@ struct BodyUpsample {
         f.init(W, a.H, (unsigned)rows, max(1u, FlatRows::kMaxValues / W), (unsigned)GW, 1);
         for (int64_t it = gw; it < f.items(); it += GW) {
             const int64_t g0 = it * f.R, g1 = min(g0 + (int64_t)f.R, rows);
-            flat_item(a, f, (unsigned)g0, (unsigned)(g1 - g0) * W, FlatGlobal{a.x + g0 * W});
+            flat_item(a, f, (unsigned)g0, (unsigned)g0 % f.H, (unsigned)(g1 - g0) * W, FlatGlobal{a.x + g0 * W});
         }
     }
 
@@ -714,30 +739,33 @@ struct BodyMaxpool {
         f.init(Wo, Ho, (unsigned)rows, min(rmax, FlatRows::kMaxValues / Wo), (unsigned)GW, 1);
         WarpRing r;
         r.init(cx, 0);
-        // input values of output rows [q0, q1), halo included
-        auto copy = [&](unsigned q0, unsigned q1, unsigned &p0, unsigned &oy0, int64_t &hi) {
-            p0 = q0 / Ho;
-            oy0 = q0 - p0 * Ho;
-            const unsigned p1 = (q1 - 1) / Ho, oy1 = q1 - 1 - p1 * Ho;
-            const int64_t lo = ((int64_t)p0 * H + 2 * (int64_t)oy0 - 1) * W - 1;
-            hi = ((int64_t)p1 * H + 2 * (int64_t)oy1 + 2) * W + 1;
+        FlatCursor fc, uc;   // the fill cursor runs the ring's stages ahead
+        fc.init(f, gw, GW);
+        uc = fc;
+        // input values of the item's output rows, halo included: n rows from
+        // row c.r of plane c.p
+        auto copy = [&](const FlatCursor &c, unsigned n, int64_t &hi) {
+            const unsigned t = c.r + n - 1, pl = f.plane_of(t), oy1 = t - pl * Ho;
+            const int64_t lo = ((int64_t)c.p * H + 2 * (int64_t)c.r - 1) * W - 1;
+            hi = ((int64_t)(c.p + pl) * H + 2 * (int64_t)oy1 + 2) * W + 1;
             return FlatCopy(lo, hi, total);
         };
-        unsigned p0, oy0;
         int64_t hi;
         ring_stream(
             r, gw, GW, f.items(),
             [&](int st, int64_t it) {
-                const unsigned q0 = (unsigned)it * f.R, q1 = min(q0 + f.R, f.rows);
-                copy(q0, q1, p0, oy0, hi).fill(r, st, a.x);
+                const unsigned q0 = (unsigned)it * f.R;
+                copy(fc, min(f.R, f.rows - q0), hi).fill(r, st, a.x);
+                fc.step(Ho);
             },
             [&](unsigned char *stage, int64_t it) {
-                const unsigned q0 = (unsigned)it * f.R, q1 = min(q0 + f.R, f.rows);
-                const FlatCopy k = copy(q0, q1, p0, oy0, hi);
+                const unsigned q0 = (unsigned)it * f.R, n = min(f.R, f.rows - q0);
+                const FlatCopy k = copy(uc, n, hi);
                 k.patch(stage, a.x, hi, total, r.lane);
-                const int64_t first = ((int64_t)p0 * H + 2 * (int64_t)oy0) * W;
-                flat_item(a, f, oy0, (q1 - q0) * Wo, a.y + (int64_t)q0 * Wo,
+                const int64_t first = ((int64_t)uc.p * H + 2 * (int64_t)uc.r) * W;
+                flat_item(a, f, uc.r, n * Wo, a.y + (int64_t)q0 * Wo,
                           FlatStage{reinterpret_cast<const float *>(stage) + (first - k.base)});
+                uc.step(Ho);
             });
         r.finish();
         return true;
