@@ -266,7 +266,11 @@ struct WarpRing {
     }
     // All lanes of the warp call this, after available() held.  Stages are
     // 128-byte multiples from a 128-byte aligned start, so every stage is a
-    // valid bulk-copy destination.
+    // valid bulk-copy destination.  The bytes may hold what an earlier kernel
+    // of the interval stored or read with ordinary accesses (counters,
+    // staging slots, values patched into a stage): its interval barrier
+    // orders those before this warp, and the proxy fence orders them before
+    // the copies that fill() issues.
     __device__ void init(const Ctx &c, size_t off, unsigned long long limit = 2000000000ull)
     {
         const int nw = c.nthreads >> 5, w = c.tid >> 5;
@@ -282,6 +286,7 @@ struct WarpRing {
             for (int s = 0; s < stages; ++s)
                 asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bars + 8u * s) : "memory");
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+            refill_fence();
         }
         __syncwarp();
     }
@@ -302,7 +307,8 @@ struct WarpRing {
                      ::"r"(dst), "l"(src), "r"(n), "r"(bars + 8u * s)
                      : "memory");
     }
-    // Lane 0, before refilling a stage the warp has read: order those reads
+    // Lane 0, before (re)filling a stage: order the ordinary accesses to it
+    // that came before, this warp's and those a barrier ordered before it,
     // before the copy engine's writes.
     __device__ void refill_fence() const { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
