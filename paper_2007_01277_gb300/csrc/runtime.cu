@@ -635,7 +635,8 @@ hf_status nway_params(const hf_fused_t *f, const void *const *args, int want, Nw
     return HF_OK;
 }
 
-// Plans a 2-way fused launch.
+// Plans a 2-way fused launch; uargs in the caller's order, the low interval's
+// kernel first (the compiled instance may have its bodies the other way).
 hf_status pair_plan(const hf_fused_t *f, const void *const *uargs, int want, LaunchPlan *plan)
 {
     const int threads[2] = {f->n_low, f->n_high};
@@ -916,7 +917,7 @@ static hf_status launch_impl(hf_fused f, const void *const *args, int grid, void
         if (s) return s;
         const void *iargs[2] = {f->low_is_a ? args[0] : args[1], f->low_is_a ? args[1] : args[0]};
         LaunchPlan plan;
-        s = pair_plan(f, iargs, grid, &plan);
+        s = pair_plan(f, args, grid, &plan);
         if (s) return s;
         PairLaunch L{iargs, f->n_low / 32, f->n_low, f->n_high, plan.off[1], plan.smem, f->low_is_a,
                      plan.grid, f->d0, hf::error_word(), {plan.ring_stage[0], plan.ring_stage[1]},
@@ -967,8 +968,7 @@ hf_status hf_query(hf_fused f, const void *const *args, hf_fused_info *info)
     if (!f || !args || !info) return fail(HF_ERR_INVALID, "NULL argument");
     LaunchPlan plan;
     if (!f->nway) {
-        const void *iargs[2] = {f->low_is_a ? args[0] : args[1], f->low_is_a ? args[1] : args[0]};
-        hf_status s = pair_plan(f, iargs, 0, &plan);
+        hf_status s = pair_plan(f, args, 0, &plan);
         if (s) return s;
     } else {
         static thread_local NwayParams p;
