@@ -79,6 +79,39 @@ struct FlatRows {
     __device__ unsigned plane_of(unsigned t) const { return H <= 1024 ? (t * mh) >> 21 : (t >= H ? 1u : 0u); }
 };
 
+// The items of the flat path without a ring: R rows as above, or, where that
+// is one row (long rows, or fewer rows than warps), runs of `cols` columns of
+// one, so that a few long rows keep every warp busy: a run is about a warp's
+// share, in whole steps of 32 columns, and 256 at most, as enough runs are as
+// even as longer ones.  One row of 1000003 values on a warp of its own took
+// 6160 / 3770 / 19600 us (upsample / max pool / im2col), as runs 7.6 / 5.6 /
+// 15.6 (one thread per output 25.6 / 5.1 / 43).
+struct FlatRuns {
+    unsigned per_row, cols;   // runs of a row, columns of each
+    int64_t items;
+    __device__ void init(const FlatRows &f, int64_t warps)
+    {
+        per_row = 1;
+        cols = f.R * f.W;
+        if (f.R == 1) {
+            const int64_t each = ((int64_t)f.rows * f.W + warps - 1) / warps;
+            const unsigned most = (unsigned)(each < 256 ? (each + 31) / 32 * 32 : 256);
+            per_row = (f.W + most - 1) / most;
+            cols = (f.W + 32 * per_row - 1) / (32 * per_row) * 32;
+        }
+        items = (int64_t)f.items() * per_row;
+    }
+    // first row of item it, and its pixels from .. upto counted from there
+    __device__ unsigned item(const FlatRows &f, int64_t it, unsigned &from, unsigned &upto) const
+    {
+        const int64_t q = per_row == 1 ? it : it / per_row;
+        const unsigned g = (unsigned)q * f.R;
+        from = (unsigned)(it - q * per_row) * cols;
+        upto = min(min(f.R, f.rows - g) * f.W, from + cols);
+        return g;
+    }
+};
+
 // Plane p and row r in it of the first row of a warp's items it, it + step,
 // ..., advanced without divisions: in items of few pixels, as max pool's two
 // rows of 74, those were a fifth of the instructions (upsample 8x64x75x75 +
@@ -387,17 +420,18 @@ struct BodyUpsample {
         return true;
     }
 
-    // One item of the flat path: pixel i gives the outputs (2r, 2r+1) x
-    // (2c, 2c+1); in memory they start at 4*i - 2*c from the item's first.
+    // One item of the flat path, its pixels from .. n - 1: pixel i gives the
+    // outputs (2r, 2r+1) x (2c, 2c+1); in memory they start at 4*i - 2*c from
+    // the item's first.
     template <class Get>
     static __device__ __forceinline__ void flat_item(const Args &a, const FlatRows &f, unsigned g0, unsigned r0,
-                                                     unsigned n, const Get &get)
+                                                     unsigned from, unsigned n, const Get &get)
     {
         const int W = (int)f.W;
         float *y0 = a.y + 4 * (int64_t)g0 * W;
         const bool y8 = (reinterpret_cast<uintptr_t>(a.y) & 7u) == 0;
 #pragma unroll 2
-        for (unsigned i = lane_id(); i < n; i += 32) {
+        for (unsigned i = from + lane_id(); i < n; i += 32) {
             const unsigned lr = f.row_of(i), c = i - lr * f.W, t = r0 + lr;
             const unsigned r = t - f.plane_of(t) * f.H;
             const bool le = c == 0, re = c == f.W - 1, te = r == 0, be = r == f.H - 1;
@@ -448,7 +482,7 @@ struct BodyUpsample {
                 const int64_t g0 = it * f.R, g1 = min(g0 + (int64_t)f.R, rows);
                 const FlatCopy k = copy(it);
                 k.patch(stage, a.x, (g1 + 1) * W + 1, total, r.lane);
-                flat_item(a, f, (unsigned)g0, uc.r, (unsigned)(g1 - g0) * W,
+                flat_item(a, f, (unsigned)g0, uc.r, 0, (unsigned)(g1 - g0) * W,
                           FlatStage{reinterpret_cast<const float *>(stage) + (g0 * W - k.base)});
                 uc.step(f.H);
             });
@@ -465,9 +499,12 @@ struct BodyUpsample {
         const unsigned W = (unsigned)a.W;
         FlatRows f;
         f.init(W, a.H, (unsigned)rows, max(1u, FlatRows::kMaxValues / W), (unsigned)GW, 1);
-        for (int64_t it = gw; it < f.items(); it += GW) {
-            const int64_t g0 = it * f.R, g1 = min(g0 + (int64_t)f.R, rows);
-            flat_item(a, f, (unsigned)g0, (unsigned)g0 % f.H, (unsigned)(g1 - g0) * W, FlatGlobal{a.x + g0 * W});
+        FlatRuns u;
+        u.init(f, GW);
+        for (int64_t it = gw; it < u.items; it += GW) {
+            unsigned from, upto;
+            const unsigned g0 = u.item(f, it, from, upto);
+            flat_item(a, f, g0, g0 % f.H, from, upto, FlatGlobal{a.x + (int64_t)g0 * W});
         }
     }
 
@@ -689,21 +726,21 @@ struct BodyMaxpool {
         return true;
     }
 
-    // One item of the flat path: its pixels are output pixels (W and H of f
-    // those of the output), get(0) is column 0 of the window centre of the
+    // One item of the flat path, its pixels from .. n - 1: output pixels (W and
+    // H of f those of the output), get(0) is column 0 of the window centre of the
     // item's first row, which is row oy0 of its plane.  The order of the
     // maxima is the strips'; where W or an alignment rules strips out a NaN
     // never wins (`clean`), as in one running maximum over the window.
     template <class Get>
-    static __device__ __forceinline__ void flat_item(const Args &a, const FlatRows &f, unsigned oy0, unsigned n,
-                                                     float *y0, const Get &get)
+    static __device__ __forceinline__ void flat_item(const Args &a, const FlatRows &f, unsigned oy0, unsigned from,
+                                                     unsigned n, float *y0, const Get &get)
     {
         const int W = a.W;
         const unsigned H = (unsigned)a.H;
         const bool clean = (a.W & 3) != 0 || !aligned16(a.x) || !aligned16(a.y);
         const float ninf = -__int_as_float(0x7f800000);
 #pragma unroll 2
-        for (unsigned i = lane_id(); i < n; i += 32) {
+        for (unsigned i = from + lane_id(); i < n; i += 32) {
             const unsigned lr = f.row_of(i), ox = i - lr * f.W, t = oy0 + lr;
             const unsigned p = f.plane_of(t), oy = t - p * f.H;
             // input row 2*oy of plane p, counted from input row 2*oy0 of the
@@ -763,7 +800,7 @@ struct BodyMaxpool {
                 const FlatCopy k = copy(uc, n, hi);
                 k.patch(stage, a.x, hi, total, r.lane);
                 const int64_t first = ((int64_t)uc.p * H + 2 * (int64_t)uc.r) * W;
-                flat_item(a, f, uc.r, n * Wo, a.y + (int64_t)q0 * Wo,
+                flat_item(a, f, uc.r, 0, n * Wo, a.y + (int64_t)q0 * Wo,
                           FlatStage{reinterpret_cast<const float *>(stage) + (first - k.base)});
                 uc.step(Ho);
             });
@@ -781,10 +818,12 @@ struct BodyMaxpool {
         const int64_t gw = (int64_t)cx.block * nw + (cx.tid >> 5), GW = (int64_t)cx.grid * nw;
         FlatRows f;
         f.init(Wo, Ho, (unsigned)rows, max(1u, FlatRows::kMaxValues / Wo), (unsigned)GW, 1);
-        for (int64_t it = gw; it < f.items(); it += GW) {
-            const unsigned q0 = (unsigned)it * f.R, q1 = min(q0 + f.R, f.rows);
-            const unsigned p0 = q0 / Ho, oy0 = q0 - p0 * Ho;
-            flat_item(a, f, oy0, (q1 - q0) * Wo, a.y + (int64_t)q0 * Wo,
+        FlatRuns u;
+        u.init(f, GW);
+        for (int64_t it = gw; it < u.items; it += GW) {
+            unsigned from, upto;
+            const unsigned q0 = u.item(f, it, from, upto), p0 = q0 / Ho, oy0 = q0 - p0 * Ho;
+            flat_item(a, f, oy0, from, upto, a.y + (int64_t)q0 * Wo,
                       FlatGlobal{a.x + ((int64_t)p0 * H + 2 * (int64_t)oy0) * W});
         }
     }
@@ -1022,15 +1061,16 @@ struct BodyIm2col {
         return true;
     }
 
-    // One item of the flat path, VEC consecutive pixels per lane.  Shifted
+    // One item of the flat path, its pixels from .. n - 1, VEC consecutive ones
+    // per lane.  Shifted
     // copy k of pixel i lies at k*HW + i of its plane's output, so a warp's
     // stores are contiguous for any W; VEC == 4 (planes of 16-byte
     // multiples, items that start on one) makes them 128-bit and reads
     // three times six values for four pixels -- in one 128-bit and two
     // 32-bit loads where the rows are 16-byte multiples too.
     template <int VEC, class Get>
-    static __device__ __forceinline__ void flat_item(const Args &a, const FlatRows &f, unsigned g0, unsigned n,
-                                                     const Get &get)
+    static __device__ __forceinline__ void flat_item(const Args &a, const FlatRows &f, unsigned g0, unsigned from,
+                                                     unsigned n, const Get &get)
     {
         const int W = (int)f.W;
         const int64_t HW = (int64_t)f.H * W;
@@ -1039,7 +1079,7 @@ struct BodyIm2col {
         float *o0 = a.col + ((int64_t)p0 * 9 * HW + (int64_t)r0 * W);
         if constexpr (VEC == 4)
             if ((W & 3) == 0) {   // the four pixels are of one row
-                for (unsigned i = 4 * lane_id(); i < n; i += 128) {
+                for (unsigned i = from + 4 * lane_id(); i < n; i += 128) {
                     const unsigned lr = f.row_of(i), t = r0 + lr, p = f.plane_of(t);
                     const unsigned c = i - lr * f.W, r = t - p * f.H;
                     const bool le = c == 0, re = c + 4 == f.W;
@@ -1057,7 +1097,7 @@ struct BodyIm2col {
                 }
                 return;
             }
-        for (unsigned i = VEC * lane_id(); i < n; i += 32 * VEC) {
+        for (unsigned i = from + VEC * lane_id(); i < n; i += 32 * VEC) {
             const unsigned lr = f.row_of(i), t = r0 + lr;
             const unsigned p = f.plane_of(t);
             unsigned c = i - lr * f.W, r = t - p * f.H;
@@ -1135,7 +1175,7 @@ struct BodyIm2col {
                 const int64_t g0 = it * f.R, g1 = min(g0 + (int64_t)f.R, rows);
                 const FlatCopy k = copy(it);
                 k.patch(stage, a.x, (g1 + 1) * W + 1, total, r.lane);
-                flat_item<VEC>(a, f, (unsigned)g0, (unsigned)(g1 - g0) * W,
+                flat_item<VEC>(a, f, (unsigned)g0, 0, (unsigned)(g1 - g0) * W,
                                FlatStage{reinterpret_cast<const float *>(stage) + (g0 * W - k.base)});
             });
         r.finish();
@@ -1151,9 +1191,12 @@ struct BodyIm2col {
         const unsigned W = (unsigned)a.W;
         FlatRows f;
         f.init(W, a.H, (unsigned)rows, max(1u, FlatRows::kMaxValues / W), (unsigned)GW, 1);
-        for (int64_t it = gw; it < f.items(); it += GW) {
-            const int64_t g0 = it * f.R, g1 = min(g0 + (int64_t)f.R, rows);
-            flat_item<1>(a, f, (unsigned)g0, (unsigned)(g1 - g0) * W, FlatGlobal{a.x + g0 * W});
+        FlatRuns u;
+        u.init(f, GW);
+        for (int64_t it = gw; it < u.items; it += GW) {
+            unsigned from, upto;
+            const unsigned g0 = u.item(f, it, from, upto);
+            flat_item<1>(a, f, g0, from, upto, FlatGlobal{a.x + (int64_t)g0 * W});
         }
     }
 
