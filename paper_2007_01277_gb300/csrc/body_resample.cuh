@@ -570,10 +570,11 @@ struct BodyMaxpool {
     // 32 / 40 / 56 / 64 columns took 74 / 43 / 28 / 25 / 22 / 21 us alone,
     // the flat path 22 / 22 / 21 / 22 / 22 / 21 (at W = 112 strips 18, flat 21).
     static constexpr int kStripCols = 64;
-    static __host__ __device__ bool strips(const Args &a)
+    static __host__ __device__ bool rows16(const Args &a)
     {
-        return (a.W & 3) == 0 && a.W >= kStripCols && aligned16(a.x) && aligned16(a.y);
+        return (a.W & 3) == 0 && aligned16(a.x) && aligned16(a.y);
     }
+    static __host__ __device__ bool strips(const Args &a) { return rows16(a) && a.W >= kStripCols; }
     // a strip's rows (W <= 128) or a flat item's arrive as one bulk copy
     static __host__ bool uses_ring(const Args &a)
     {
@@ -857,10 +858,13 @@ struct BodyMaxpool {
     static __device__ void run(const Args &a, const Ctx &cx)
     {
         if ((int64_t)a.P * a.H * a.W == 0) return;
-        if (strips(a)) {
+        // 16-byte rows keep the strips' order of maxima, so that a NaN counts
+        // alike whatever the tensor's size
+        const bool flat = flat_range((int64_t)a.P * a.H, a.W, cx);
+        if (strips(a) || (!flat && rows16(a))) {
             if (a.W <= 128 && a.H >= 2 && WarpRing::available(cx, 0) && run_ring(a, cx)) return;
             run_vec(a, cx);
-        } else if (flat_range((int64_t)a.P * a.H, a.W, cx)) {
+        } else if (flat) {
             if (!flat_ring(a, cx)) flat_global(a, cx);
         } else {
             run_scalar(a, cx);
