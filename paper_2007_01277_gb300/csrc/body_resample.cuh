@@ -121,11 +121,15 @@ struct FlatCursor {
     unsigned p, r, dp, dr;
     __device__ void init(const FlatRows &f, int64_t it, int64_t step)
     {
-        const uint64_t row = it < (int64_t)f.items() ? (uint64_t)it * f.R : 0, d = (uint64_t)step * f.R;
-        p = (unsigned)(row / f.H);
-        r = (unsigned)(row - (uint64_t)p * f.H);
-        dp = (unsigned)(d / f.H);   // beyond 32 bits only where no second item exists
-        dr = (unsigned)(d - d / f.H * f.H);
+        // 32-bit divisions: a step past every row stands for all longer ones,
+        // which have no second item
+        const unsigned row = it < (int64_t)f.items() ? (unsigned)it * f.R : 0;
+        const int64_t far = step * f.R;
+        const unsigned d = far < (1ll << 31) ? (unsigned)far : 1u << 31;
+        p = row / f.H;
+        r = row - p * f.H;
+        dp = d / f.H;
+        dr = d - dp * f.H;
     }
     __device__ void step(unsigned H)
     {
@@ -182,6 +186,15 @@ __device__ __forceinline__ bool flat_range(int64_t rows, int64_t W, const Ctx &c
 {
     return rows < ((int64_t)1 << 31) && W < ((int64_t)1 << 29) && (int64_t)cx.grid * (cx.nthreads >> 5) < ((int64_t)1 << 31);
 }
+// At most `each` of something per thread, or per warp, of the grid.
+__device__ __forceinline__ bool per_thread(int64_t n, const Ctx &cx, int each)
+{
+    return n <= (int64_t)each * cx.grid * cx.nthreads;
+}
+__device__ __forceinline__ bool per_warp(int64_t n, const Ctx &cx, int each)
+{
+    return n <= (int64_t)each * cx.grid * (cx.nthreads >> 5);
+}
 // Floats of a stage that an item's halo and the rounding take: base is up to
 // three below lo, the copy's end up to three past hi.
 constexpr unsigned kFlatPad = 8;
@@ -203,6 +216,7 @@ struct BodyUpsample {
     static constexpr int kRingRows = 6;
     static constexpr bool kRingItem = true;
     static constexpr unsigned kRingMinBytes = 4096;   // the stage: one item
+    static constexpr int kSingleBlock = 768;          // 90 registers otherwise, 640 threads
 
     // Which path: 16-byte rows of 64 values or more go to strips of whole
     // rows (four columns a lane), the others to the flat path.  Strips leave
@@ -213,7 +227,14 @@ struct BodyUpsample {
     // rows with their halo still fit a flat item's: 57 us on registers, 51
     // flat (W = 224, four warps an SM; 39 and 37 us at full occupancy).
     // Longer ones keep the register path (W = 400: 39 us, 47 flat).
+    // Small tensors cannot repay the flat path's start (a dozen divisions and
+    // the ring): up to kFewRows rows per warp go to strips (24 warps an SM,
+    // 2000 rows of 16 / 60 columns 4.0 / 4.1 us, flat 4.4 / 5.1; 32000 rows of
+    // 16 columns, 9 a warp, 8.4 and 5.7), and where those are ruled out up to
+    // kFewOutputs outputs per thread to a thread each (60 rows of 75 columns
+    // 2.8 us, flat 3.9; 2000 rows 7.2 and 5.2).
     static constexpr int kStripCols = 64;
+    static constexpr int kFewOutputs = 1, kFewRows = 5;
     static __host__ __device__ bool rows16(const Args &a)
     {
         return (a.W & 3) == 0 && aligned16(a.x) && aligned16(a.y);
@@ -508,7 +529,7 @@ struct BodyUpsample {
         }
     }
 
-    // One thread per output: tensors of 2^31 rows or more.
+    // One thread per output: few outputs, and tensors of 2^31 rows or more.
     static __device__ void run_scalar(const Args &a, const Ctx &cx)
     {
         const int H = a.H, W = a.W, Ho = 2 * H, Wo = 2 * W;
@@ -540,13 +561,13 @@ struct BodyUpsample {
     static __device__ void run(const Args &a, const Ctx &cx)
     {
         if ((int64_t)a.P * a.H * a.W == 0) return;
-        const bool flat = flat_range((int64_t)a.P * a.H, a.W, cx);
-        if (strips(a)) {
-            if (a.W <= 128 && WarpRing::available(cx, 0) && run_ring(a, cx)) return;
-        } else if (flat && flat_ring(a, cx)) {
-            return;
-        }
-        if (a.W >= kStripCols && rows16(a)) run_vec(a, cx);
+        const int64_t rows = (int64_t)a.P * a.H;
+        const bool vec = rows16(a);
+        const bool flat = flat_range(rows, a.W, cx) &&
+                          !(vec ? per_warp(rows, cx, kFewRows) : per_thread(4 * rows * a.W, cx, kFewOutputs));
+        if (flat && !strips(a) && flat_ring(a, cx)) return;
+        if (vec && a.W <= 128 && WarpRing::available(cx, 0) && run_ring(a, cx)) return;
+        if (vec && (a.W >= kStripCols || !flat)) run_vec(a, cx);
         else if (flat) flat_global(a, cx);
         else run_scalar(a, cx);
     }
@@ -569,7 +590,16 @@ struct BodyMaxpool {
     // lanes idle below 128 columns: 2^23 values in images of W = 8 / 16 /
     // 32 / 40 / 56 / 64 columns took 74 / 43 / 28 / 25 / 22 / 21 us alone,
     // the flat path 22 / 22 / 21 / 22 / 22 / 21 (at W = 112 strips 18, flat 21).
+    // Small tensors cannot repay the flat path's start: few_rows() per warp go
+    // to strips -- the closer the rows come to 64 columns the more (24 warps
+    // an SM, 4000 rows of 8 columns 3.9 us, flat 4.7; 37000 rows of 56, 10 a
+    // warp, 7.6 and 9.6; 16 warps, 35000 rows of 60, 14 a warp, 7.2 and 8.2;
+    // but 58 a warp 12.1 and 10.6) -- and where those are ruled out up to two
+    // outputs per thread to a thread each (2000 rows of 38 outputs 3.2 us,
+    // flat 5.5), ten where no ring holds three rows (224 rows of 501, nine a
+    // thread, 9.8 us, flat 11.0; 27 a thread 26 and 16).
     static constexpr int kStripCols = 64;
+    static __device__ int few_rows(int W) { return W >= 60 ? 32 : W >= 48 ? 12 : 5; }
     static __host__ __device__ bool rows16(const Args &a)
     {
         return (a.W & 3) == 0 && aligned16(a.x) && aligned16(a.y);
@@ -579,7 +609,12 @@ struct BodyMaxpool {
     static __host__ bool uses_ring(const Args &a)
     {
         if ((int64_t)a.P * a.H * a.W <= 0) return false;
-        return strips(a) ? a.W <= 128 && a.H >= 2 : aligned16(a.x) && 3u * a.W + kFlatPad <= kRingMinBytes / 4;
+        return strips(a) ? a.W <= 128 && a.H >= 2 : ring_rows(a);
+    }
+    // three rows and the rounding fit a stage: what a flat item needs
+    static __host__ __device__ bool ring_rows(const Args &a)
+    {
+        return aligned16(a.x) && 3u * a.W + kFlatPad <= kRingMinBytes / 4;
     }
 
     static __host__ size_t workspace_bytes(const Args &) { return 0; }
@@ -829,7 +864,7 @@ struct BodyMaxpool {
         }
     }
 
-    // One thread per output: tensors of 2^31 rows or more.
+    // One thread per output: few outputs, and tensors of 2^31 rows or more.
     static __device__ void run_scalar(const Args &a, const Ctx &cx)
     {
         const int H = a.H, W = a.W, Ho = (H - 1) / 2 + 1, Wo = (W - 1) / 2 + 1;
@@ -858,10 +893,14 @@ struct BodyMaxpool {
     static __device__ void run(const Args &a, const Ctx &cx)
     {
         if ((int64_t)a.P * a.H * a.W == 0) return;
-        // 16-byte rows keep the strips' order of maxima, so that a NaN counts
-        // alike whatever the tensor's size
-        const bool flat = flat_range((int64_t)a.P * a.H, a.W, cx);
-        if (strips(a) || (!flat && rows16(a))) {
+        const int64_t rows = (int64_t)a.P * ((a.H - 1) / 2 + 1);
+        const bool vec = rows16(a);
+        const bool flat = flat_range((int64_t)a.P * a.H, a.W, cx) &&
+                          !(vec ? per_warp(rows, cx, few_rows(a.W))
+                                : per_thread(rows * ((a.W - 1) / 2 + 1), cx, ring_rows(a) ? 2 : 10));
+        // not flat: also past 2^31 rows, where 16-byte rows keep the strips'
+        // order of maxima, so that a NaN counts alike whatever the size
+        if (vec && (a.W >= kStripCols || !flat)) {
             if (a.W <= 128 && a.H >= 2 && WarpRing::available(cx, 0) && run_ring(a, cx)) return;
             run_vec(a, cx);
         } else if (flat) {
@@ -892,6 +931,11 @@ struct BodyIm2col {
     // 100 bytes of spills and 5 to 11 % (histogram + im2col).
     static constexpr int kRingRows = 14;   // rows of a strip item
     static constexpr int kStripCols = 56;
+    // Up to as many outputs per thread the flat path's start (a dozen
+    // divisions and the ring) costs more than a thread per output: 60 rows of
+    // 75 columns, 1 a thread, 3.3 us, flat 5.2; 60 of 337, 5 a thread, 4.3 and
+    // 6.4; 300 of 112, 8 a thread, 5.6 and 3.9.
+    static constexpr int kFewOutputs = 5;
     static constexpr bool kRingItem = true;
     static constexpr unsigned kRingMinBytes = 4096;   // the stage: one item
     static __host__ bool uses_ring(const Args &a)
@@ -1204,7 +1248,7 @@ struct BodyIm2col {
         }
     }
 
-    // One thread per output: tensors of 2^31 rows or more.
+    // One thread per output: few outputs, and tensors of 2^31 rows or more.
     static __device__ void run_scalar(const Args &a, const Ctx &cx)
     {
         const int H = a.H, W = a.W;
@@ -1229,16 +1273,17 @@ struct BodyIm2col {
     static __device__ __forceinline__ void run_as(const Args &a, const Ctx &cx)
     {
         if ((int64_t)a.N * a.C * a.H * a.W == 0) return;
-        const bool flat = flat_range((int64_t)a.N * a.C * a.H, a.W, cx);
-        if (STRIPS && cx.nthreads == 32 && (a.W & 3) == 0 && a.W >= kStripCols && a.W <= 64 && aligned16(a.x) &&
-            aligned16(a.col) && WarpRing::available(cx, 0) && run_ring(a, cx))
+        const bool rows16 = (a.W & 3) == 0 && a.W <= 64 && aligned16(a.x) && aligned16(a.col);
+        const bool flat = flat_range((int64_t)a.N * a.C * a.H, a.W, cx) &&
+                          (rows16 || !per_thread(9 * (int64_t)a.N * a.C * a.H * a.W, cx, kFewOutputs));
+        if (STRIPS && cx.nthreads == 32 && rows16 && a.W >= kStripCols && WarpRing::available(cx, 0) && run_ring(a, cx))
             return;
         if (flat) {
             const bool v4 = a.W >= 4 && ((int64_t)a.H * a.W & 3) == 0 && aligned16(a.col);
             if (v4 && flat_ring<4>(a, cx)) return;
             if (flat_ring<1>(a, cx)) return;
         }
-        if ((a.W & 3) == 0 && a.W <= 64 && aligned16(a.x) && aligned16(a.col)) run_vec(a, cx);
+        if (rows16) run_vec(a, cx);
         else if (flat) flat_global(a, cx);
         else run_scalar(a, cx);
     }

@@ -22,7 +22,7 @@ const Instance *nway_table(int *n)
 template <class B>
 SingleEntry make_single()
 {
-    return SingleEntry{B::kId, reinterpret_cast<const void *>(&k_single<B>), single_full_func<B>(), &launch_single<B>};
+    return SingleEntry{B::kId, single_func<B>(), single_full_func<B>(), &launch_single<B>};
 }
 
 static const SingleEntry kSingles[] = {

@@ -67,10 +67,12 @@ __global__ void k_single(const __grid_constant__ SingleParams<B> p)
     single_body<B>(p);
 }
 
-// The same with the registers that blocks of 1024 threads leave, for bodies
-// that declare kFullBlock: launches that k_single's registers do not allow.
-template <class B>
-__global__ void __launch_bounds__(1024) k_single_full(const __grid_constant__ SingleParams<B> p)
+// The same with the registers that blocks of T threads leave: for bodies that
+// declare kSingleBlock in place of k_single (the compiler would spend registers
+// that cost larger blocks), for bodies that declare kFullBlock beside it, at
+// 1024 threads, for launches that k_single's registers do not allow.
+template <class B, int T>
+__global__ void __launch_bounds__(T) k_single_block(const __grid_constant__ SingleParams<B> p)
 {
     single_body<B>(p);
 }
@@ -80,10 +82,24 @@ struct FullBlock : std::false_type {
 template <class B>
 struct FullBlock<B, std::void_t<decltype(B::kFullBlock)>> : std::true_type {
 };
+template <class B, class = void>
+struct SingleBlock : std::false_type {
+};
+template <class B>
+struct SingleBlock<B, std::void_t<decltype(B::kSingleBlock)>> : std::true_type {
+};
+template <class B>
+const void *single_func()
+{
+    if constexpr (SingleBlock<B>::value)
+        return reinterpret_cast<const void *>(&k_single_block<B, B::kSingleBlock>);
+    else
+        return reinterpret_cast<const void *>(&k_single<B>);
+}
 template <class B>
 const void *single_full_func()
 {
-    if constexpr (FullBlock<B>::value) return reinterpret_cast<const void *>(&k_single_full<B>);
+    if constexpr (FullBlock<B>::value) return reinterpret_cast<const void *>(&k_single_block<B, 1024>);
     return nullptr;
 }
 
@@ -337,8 +353,8 @@ const Instance *nway_table(int *n);
 // Standalone kernels: one per body, no register bound.
 struct SingleEntry {
     int body;
-    const void *func;        // k_single
-    const void *func_full;   // k_single_full, or nullptr
+    const void *func;        // k_single, or k_single_block
+    const void *func_full;   // k_single_block of 1024 threads, or nullptr
     cudaError_t (*launch)(const void *func, const void *args, int threads, int grid, unsigned smem, unsigned *err,
                           unsigned ring_stage, int ring_stages, cudaStream_t);
 };
