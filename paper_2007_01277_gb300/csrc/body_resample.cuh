@@ -79,39 +79,6 @@ struct FlatRows {
     __device__ unsigned plane_of(unsigned t) const { return H <= 1024 ? (t * mh) >> 21 : (t >= H ? 1u : 0u); }
 };
 
-// The items of the flat path without a ring: R rows as above, or, where that
-// is one row (long rows, or fewer rows than warps), runs of `cols` columns of
-// one, so that a few long rows keep every warp busy: a run is about a warp's
-// share, in whole steps of 32 columns, and 256 at most, as enough runs are as
-// even as longer ones.  One row of 1000003 values on a warp of its own took
-// 6160 / 3770 / 19600 us (upsample / max pool / im2col), as runs 7.6 / 5.6 /
-// 15.6 (one thread per output 25.6 / 5.1 / 43).
-struct FlatRuns {
-    unsigned per_row, cols;   // runs of a row, columns of each
-    int64_t items;
-    __device__ void init(const FlatRows &f, int64_t warps)
-    {
-        per_row = 1;
-        cols = f.R * f.W;
-        if (f.R == 1) {
-            const int64_t each = ((int64_t)f.rows * f.W + warps - 1) / warps;
-            const unsigned most = (unsigned)(each < 256 ? (each + 31) / 32 * 32 : 256);
-            per_row = (f.W + most - 1) / most;
-            cols = (f.W + 32 * per_row - 1) / (32 * per_row) * 32;
-        }
-        items = (int64_t)f.items() * per_row;
-    }
-    // first row of item it, and its pixels from .. upto counted from there
-    __device__ unsigned item(const FlatRows &f, int64_t it, unsigned &from, unsigned &upto) const
-    {
-        const int64_t q = per_row == 1 ? it : it / per_row;
-        const unsigned g = (unsigned)q * f.R;
-        from = (unsigned)(it - q * per_row) * cols;
-        upto = min(min(f.R, f.rows - g) * f.W, from + cols);
-        return g;
-    }
-};
-
 // Plane p and row r in it of the first row of a warp's items it, it + step,
 // ..., advanced without divisions: in items of few pixels, as max pool's two
 // rows of 74, those were a fifth of the instructions (upsample 8x64x75x75 +
@@ -121,15 +88,11 @@ struct FlatCursor {
     unsigned p, r, dp, dr;
     __device__ void init(const FlatRows &f, int64_t it, int64_t step)
     {
-        // 32-bit divisions: a step past every row stands for all longer ones,
-        // which have no second item
-        const unsigned row = it < (int64_t)f.items() ? (unsigned)it * f.R : 0;
-        const int64_t far = step * f.R;
-        const unsigned d = far < (1ll << 31) ? (unsigned)far : 1u << 31;
-        p = row / f.H;
-        r = row - p * f.H;
-        dp = d / f.H;
-        dr = d - dp * f.H;
+        const uint64_t row = it < (int64_t)f.items() ? (uint64_t)it * f.R : 0, d = (uint64_t)step * f.R;
+        p = (unsigned)(row / f.H);
+        r = (unsigned)(row - (uint64_t)p * f.H);
+        dp = (unsigned)(d / f.H);   // beyond 32 bits only where no second item exists
+        dr = (unsigned)(d - d / f.H * f.H);
     }
     __device__ void step(unsigned H)
     {
@@ -186,14 +149,16 @@ __device__ __forceinline__ bool flat_range(int64_t rows, int64_t W, const Ctx &c
 {
     return rows < ((int64_t)1 << 31) && W < ((int64_t)1 << 29) && (int64_t)cx.grid * (cx.nthreads >> 5) < ((int64_t)1 << 31);
 }
-// At most `each` of something per thread, or per warp, of the grid.
-__device__ __forceinline__ bool per_thread(int64_t n, const Ctx &cx, int each)
+// Whether the flat path without a ring keeps enough warps busy: an item is at
+// least one row, so a tensor has `rows` items at most, and below one for every
+// `per` warps a thread per output is faster however long the rows are (one row
+// of 1000003 values on one warp: 6160 / 3770 / 19600 us for upsample / max
+// pool / im2col, a thread per output 25.6 / 5.1 / 43.3).  The lines are where
+// a warp's 32 outputs in turn (0.20 / 0.24 / 0.63 us) cost what the threads'
+// shares do (1.0 / 0.5 / 0.56 us an output).
+__device__ __forceinline__ bool enough_rows(int64_t rows, const Ctx &cx, int per)
 {
-    return n <= (int64_t)each * cx.grid * cx.nthreads;
-}
-__device__ __forceinline__ bool per_warp(int64_t n, const Ctx &cx, int each)
-{
-    return n <= (int64_t)each * cx.grid * (cx.nthreads >> 5);
+    return rows * per >= (int64_t)cx.grid * (cx.nthreads >> 5);
 }
 // Floats of a stage that an item's halo and the rounding take: base is up to
 // three below lo, the copy's end up to three past hi.
@@ -216,28 +181,32 @@ struct BodyUpsample {
     static constexpr int kRingRows = 6;
     static constexpr bool kRingItem = true;
     static constexpr unsigned kRingMinBytes = 4096;   // the stage: one item
-    static constexpr int kSingleBlock = 768;          // 90 registers otherwise, 640 threads
 
     // Which path: 16-byte rows of 64 values or more go to strips of whole
     // rows (four columns a lane), the others to the flat path.  Strips leave
     // lanes idle below 128 columns: 2^23 values in images of W = 8 / 16 /
     // 32 / 40 / 56 / 64 columns took 181 / 83 / 49 / 41 / 35 / 33 us alone,
-    // the flat path 37 / 35 / 34 / 36 / 35 / 35.
+    // the flat path 37 / 35 / 34 / 36 / 35 / 35 (112: 37 and 35).  In a narrow
+    // interval the flat path's cost does not depend on W and a strip's falls
+    // with it: 2^22 values with one warp an SM, W = 32 / 40 / 48 / 56 / 60 / 64 /
+    // 96 / 112, strips 156 / 116 / 94 / 86 / 76 / 72 / 48 / 43 us, flat 65 to 70.
     // Rows of 129 to 252 columns are too long for a strip's stage, but two
     // rows with their halo still fit a flat item's: 57 us on registers, 51
     // flat (W = 224, four warps an SM; 39 and 37 us at full occupancy).
     // Longer ones keep the register path (W = 400: 39 us, 47 flat).
-    // Small tensors cannot repay the flat path's start (a dozen divisions and
-    // the ring): up to kFewRows rows per warp go to strips (24 warps an SM,
-    // 2000 rows of 16 / 60 columns 4.0 / 4.1 us, flat 4.4 / 5.1; 32000 rows of
-    // 16 columns, 9 a warp, 8.4 and 5.7), and where those are ruled out up to
-    // kFewOutputs outputs per thread to a thread each (60 rows of 75 columns
-    // 2.8 us, flat 3.9; 2000 rows 7.2 and 5.2).
+    // Small tensors of other rows cannot repay the flat path's start (a dozen
+    // divisions and the ring): up to kFewOutputs outputs per thread go to a
+    // thread each (60 rows of 75 columns 2.8 us, flat 3.9; 2000 rows 7.2 and
+    // 5.2).
     static constexpr int kStripCols = 64;
-    static constexpr int kFewOutputs = 1, kFewRows = 5;
+    static constexpr int kFewOutputs = 1;
     static __host__ __device__ bool rows16(const Args &a)
     {
         return (a.W & 3) == 0 && aligned16(a.x) && aligned16(a.y);
+    }
+    static __host__ __device__ bool small(const Args &a, int64_t threads)   // of the grid
+    {
+        return !rows16(a) && 4 * (int64_t)a.P * a.H * a.W <= kFewOutputs * threads;
     }
     static __host__ __device__ bool strips(const Args &a)
     {
@@ -441,18 +410,17 @@ struct BodyUpsample {
         return true;
     }
 
-    // One item of the flat path, its pixels from .. n - 1: pixel i gives the
-    // outputs (2r, 2r+1) x (2c, 2c+1); in memory they start at 4*i - 2*c from
-    // the item's first.
+    // One item of the flat path: pixel i gives the outputs (2r, 2r+1) x
+    // (2c, 2c+1); in memory they start at 4*i - 2*c from the item's first.
     template <class Get>
     static __device__ __forceinline__ void flat_item(const Args &a, const FlatRows &f, unsigned g0, unsigned r0,
-                                                     unsigned from, unsigned n, const Get &get)
+                                                     unsigned n, const Get &get)
     {
         const int W = (int)f.W;
         float *y0 = a.y + 4 * (int64_t)g0 * W;
         const bool y8 = (reinterpret_cast<uintptr_t>(a.y) & 7u) == 0;
 #pragma unroll 2
-        for (unsigned i = from + lane_id(); i < n; i += 32) {
+        for (unsigned i = lane_id(); i < n; i += 32) {
             const unsigned lr = f.row_of(i), c = i - lr * f.W, t = r0 + lr;
             const unsigned r = t - f.plane_of(t) * f.H;
             const bool le = c == 0, re = c == f.W - 1, te = r == 0, be = r == f.H - 1;
@@ -503,7 +471,7 @@ struct BodyUpsample {
                 const int64_t g0 = it * f.R, g1 = min(g0 + (int64_t)f.R, rows);
                 const FlatCopy k = copy(it);
                 k.patch(stage, a.x, (g1 + 1) * W + 1, total, r.lane);
-                flat_item(a, f, (unsigned)g0, uc.r, 0, (unsigned)(g1 - g0) * W,
+                flat_item(a, f, (unsigned)g0, uc.r, (unsigned)(g1 - g0) * W,
                           FlatStage{reinterpret_cast<const float *>(stage) + (g0 * W - k.base)});
                 uc.step(f.H);
             });
@@ -520,16 +488,14 @@ struct BodyUpsample {
         const unsigned W = (unsigned)a.W;
         FlatRows f;
         f.init(W, a.H, (unsigned)rows, max(1u, FlatRows::kMaxValues / W), (unsigned)GW, 1);
-        FlatRuns u;
-        u.init(f, GW);
-        for (int64_t it = gw; it < u.items; it += GW) {
-            unsigned from, upto;
-            const unsigned g0 = u.item(f, it, from, upto);
-            flat_item(a, f, g0, g0 % f.H, from, upto, FlatGlobal{a.x + (int64_t)g0 * W});
+        for (int64_t it = gw; it < f.items(); it += GW) {
+            const int64_t g0 = it * f.R, g1 = min(g0 + (int64_t)f.R, rows);
+            flat_item(a, f, (unsigned)g0, (unsigned)g0 % f.H, (unsigned)(g1 - g0) * W, FlatGlobal{a.x + g0 * W});
         }
     }
 
-    // One thread per output: few outputs, and tensors of 2^31 rows or more.
+    // One thread per output: few outputs, few long rows, and tensors of 2^31
+    // rows or more.
     static __device__ void run_scalar(const Args &a, const Ctx &cx)
     {
         const int H = a.H, W = a.W, Ho = 2 * H, Wo = 2 * W;
@@ -558,18 +524,48 @@ struct BodyUpsample {
         }
     }
 
+    // SMALL: with the rule on small tensors (a kernel launched alone is chosen
+    // by it before the launch).
+    template <bool SMALL, int>
+    static __device__ __forceinline__ void run_as(const Args &a, const Ctx &cx)
+    {
+        if ((int64_t)a.P * a.H * a.W == 0) return;
+        const bool vec = rows16(a);
+        bool flat = flat_range((int64_t)a.P * a.H, a.W, cx);
+        if (SMALL && small(a, (int64_t)cx.grid * cx.nthreads)) flat = false;
+        if (vec && !(flat && !strips(a))) {
+            if (a.W <= 128 && WarpRing::available(cx, 0) && run_ring(a, cx)) return;
+        } else if (flat && flat_ring(a, cx)) {
+            return;
+        }
+        if (vec && (a.W >= kStripCols || !flat)) run_vec(a, cx);
+        else if (flat && enough_rows((int64_t)a.P * a.H, cx, 12)) flat_global(a, cx);
+        else run_scalar(a, cx);
+    }
+};
+
+// The body without the flat path, launched alone where that is not the better
+// one: strips of 16-byte rows, else one thread per output.  A kernel of its
+// own, because beside the flat path the compiler's strips take up to 10 % and
+// more registers.
+struct BodyUpsamplePlain {
+    using Of = BodyUpsample;
+    using Args = Of::Args;
+    static constexpr int kId = Of::kId;
+    static __host__ bool pick(const Args &a, int, int64_t threads) { return Of::strips(a) || Of::small(a, threads); }
+    static __host__ bool uses_ring(const Args &a)
+    {
+        return (int64_t)a.P * a.H * a.W > 0 && Of::rows16(a) && a.W <= 128;
+    }
     static __device__ void run(const Args &a, const Ctx &cx)
     {
         if ((int64_t)a.P * a.H * a.W == 0) return;
-        const int64_t rows = (int64_t)a.P * a.H;
-        const bool vec = rows16(a);
-        const bool flat = flat_range(rows, a.W, cx) &&
-                          !(vec ? per_warp(rows, cx, kFewRows) : per_thread(4 * rows * a.W, cx, kFewOutputs));
-        if (flat && !strips(a) && flat_ring(a, cx)) return;
-        if (vec && a.W <= 128 && WarpRing::available(cx, 0) && run_ring(a, cx)) return;
-        if (vec && (a.W >= kStripCols || !flat)) run_vec(a, cx);
-        else if (flat) flat_global(a, cx);
-        else run_scalar(a, cx);
+        if (Of::rows16(a)) {
+            if (a.W <= 128 && WarpRing::available(cx, 0) && Of::run_ring(a, cx)) return;
+            Of::run_vec(a, cx);
+        } else {
+            Of::run_scalar(a, cx);
+        }
     }
 };
 
@@ -590,16 +586,24 @@ struct BodyMaxpool {
     // lanes idle below 128 columns: 2^23 values in images of W = 8 / 16 /
     // 32 / 40 / 56 / 64 columns took 74 / 43 / 28 / 25 / 22 / 21 us alone,
     // the flat path 22 / 22 / 21 / 22 / 22 / 21 (at W = 112 strips 18, flat 21).
-    // Small tensors cannot repay the flat path's start: few_rows() per warp go
-    // to strips -- the closer the rows come to 64 columns the more (24 warps
-    // an SM, 4000 rows of 8 columns 3.9 us, flat 4.7; 37000 rows of 56, 10 a
-    // warp, 7.6 and 9.6; 16 warps, 35000 rows of 60, 14 a warp, 7.2 and 8.2;
-    // but 58 a warp 12.1 and 10.6) -- and where those are ruled out up to two
-    // outputs per thread to a thread each (2000 rows of 38 outputs 3.2 us,
-    // flat 5.5), ten where no ring holds three rows (224 rows of 501, nine a
-    // thread, 9.8 us, flat 11.0; 27 a thread 26 and 16).
+    // With one warp an SM (2^22 values, W = 32 / 48 / 56 / 60 / 64) strips took
+    // 66 / 46 / 40 / 39 / 34 us, flat 31 / 32 / 29 / 31 / 33.  Between, where a warp has
+    // but a few items, the flat path's larger ones are less even: from 48
+    // columns on, 1 to 12 rows a warp go to strips, from 60 on 1 to 32 (24 warps
+    // an SM, 37000 rows of 56 outputs, 10 a warp, 7.6 us, flat 9.6; 16 warps,
+    // 35000 rows of 60, 14 a warp, 7.2 and 8.2; 58 a warp 12.1 and 10.6; less
+    // than one a warp 4.4 and 3.1).
+    // Small tensors of other rows cannot repay the flat path's start (a dozen
+    // divisions and the ring): up to two outputs per thread go to a thread each
+    // (2000 rows of 38 outputs 3.2 us, flat 5.5), eight where no ring holds three
+    // rows (27 a thread 26 us, flat 16).
     static constexpr int kStripCols = 64;
-    static __device__ int few_rows(int W) { return W >= 60 ? 32 : W >= 48 ? 12 : 5; }
+    static __host__ __device__ bool small(const Args &a, int64_t threads)   // of the grid
+    {
+        const int64_t rows = (int64_t)a.P * ((a.H - 1) / 2 + 1), warps = threads / 32;
+        return rows16(a) ? a.W >= 48 && rows > warps && rows <= (a.W >= 60 ? 32 : 12) * warps
+                         : rows * ((a.W - 1) / 2 + 1) <= (ring_rows(a) ? 2 : 8) * threads;
+    }
     static __host__ __device__ bool rows16(const Args &a)
     {
         return (a.W & 3) == 0 && aligned16(a.x) && aligned16(a.y);
@@ -762,21 +766,21 @@ struct BodyMaxpool {
         return true;
     }
 
-    // One item of the flat path, its pixels from .. n - 1: output pixels (W and
-    // H of f those of the output), get(0) is column 0 of the window centre of the
+    // One item of the flat path: its pixels are output pixels (W and H of f
+    // those of the output), get(0) is column 0 of the window centre of the
     // item's first row, which is row oy0 of its plane.  The order of the
     // maxima is the strips'; where W or an alignment rules strips out a NaN
     // never wins (`clean`), as in one running maximum over the window.
     template <class Get>
-    static __device__ __forceinline__ void flat_item(const Args &a, const FlatRows &f, unsigned oy0, unsigned from,
-                                                     unsigned n, float *y0, const Get &get)
+    static __device__ __forceinline__ void flat_item(const Args &a, const FlatRows &f, unsigned oy0, unsigned n,
+                                                     float *y0, const Get &get)
     {
         const int W = a.W;
         const unsigned H = (unsigned)a.H;
         const bool clean = (a.W & 3) != 0 || !aligned16(a.x) || !aligned16(a.y);
         const float ninf = -__int_as_float(0x7f800000);
 #pragma unroll 2
-        for (unsigned i = from + lane_id(); i < n; i += 32) {
+        for (unsigned i = lane_id(); i < n; i += 32) {
             const unsigned lr = f.row_of(i), ox = i - lr * f.W, t = oy0 + lr;
             const unsigned p = f.plane_of(t), oy = t - p * f.H;
             // input row 2*oy of plane p, counted from input row 2*oy0 of the
@@ -836,7 +840,7 @@ struct BodyMaxpool {
                 const FlatCopy k = copy(uc, n, hi);
                 k.patch(stage, a.x, hi, total, r.lane);
                 const int64_t first = ((int64_t)uc.p * H + 2 * (int64_t)uc.r) * W;
-                flat_item(a, f, uc.r, 0, n * Wo, a.y + (int64_t)q0 * Wo,
+                flat_item(a, f, uc.r, n * Wo, a.y + (int64_t)q0 * Wo,
                           FlatStage{reinterpret_cast<const float *>(stage) + (first - k.base)});
                 uc.step(Ho);
             });
@@ -854,17 +858,16 @@ struct BodyMaxpool {
         const int64_t gw = (int64_t)cx.block * nw + (cx.tid >> 5), GW = (int64_t)cx.grid * nw;
         FlatRows f;
         f.init(Wo, Ho, (unsigned)rows, max(1u, FlatRows::kMaxValues / Wo), (unsigned)GW, 1);
-        FlatRuns u;
-        u.init(f, GW);
-        for (int64_t it = gw; it < u.items; it += GW) {
-            unsigned from, upto;
-            const unsigned q0 = u.item(f, it, from, upto), p0 = q0 / Ho, oy0 = q0 - p0 * Ho;
-            flat_item(a, f, oy0, from, upto, a.y + (int64_t)q0 * Wo,
+        for (int64_t it = gw; it < f.items(); it += GW) {
+            const unsigned q0 = (unsigned)it * f.R, q1 = min(q0 + f.R, f.rows);
+            const unsigned p0 = q0 / Ho, oy0 = q0 - p0 * Ho;
+            flat_item(a, f, oy0, (q1 - q0) * Wo, a.y + (int64_t)q0 * Wo,
                       FlatGlobal{a.x + ((int64_t)p0 * H + 2 * (int64_t)oy0) * W});
         }
     }
 
-    // One thread per output: few outputs, and tensors of 2^31 rows or more.
+    // One thread per output: few outputs, few long rows, and tensors of 2^31
+    // rows or more.
     static __device__ void run_scalar(const Args &a, const Ctx &cx)
     {
         const int H = a.H, W = a.W, Ho = (H - 1) / 2 + 1, Wo = (W - 1) / 2 + 1;
@@ -890,23 +893,46 @@ struct BodyMaxpool {
         }
     }
 
+    // SMALL: with the rule on small tensors (a kernel launched alone is chosen
+    // by it before the launch).
+    template <bool SMALL, int>
+    static __device__ __forceinline__ void run_as(const Args &a, const Ctx &cx)
+    {
+        if ((int64_t)a.P * a.H * a.W == 0) return;
+        // not flat: also past 2^31 rows, where 16-byte rows keep the strips'
+        // order of maxima, so that a NaN counts alike whatever the size
+        const bool flat =
+            flat_range((int64_t)a.P * a.H, a.W, cx) && !(SMALL && small(a, (int64_t)cx.grid * cx.nthreads));
+        if (strips(a) || (!flat && rows16(a))) {
+            if (a.W <= 128 && a.H >= 2 && WarpRing::available(cx, 0) && run_ring(a, cx)) return;
+            run_vec(a, cx);
+            return;
+        }
+        if (flat && flat_ring(a, cx)) return;
+        // 16-byte rows are flat here, and stay so for the order of maxima
+        if (flat && (rows16(a) || enough_rows((int64_t)a.P * ((a.H - 1) / 2 + 1), cx, 2))) flat_global(a, cx);
+        else run_scalar(a, cx);
+    }
+};
+
+// The body without the flat path, as BodyUpsamplePlain.
+struct BodyMaxpoolPlain {
+    using Of = BodyMaxpool;
+    using Args = Of::Args;
+    static constexpr int kId = Of::kId;
+    static __host__ bool pick(const Args &a, int, int64_t threads) { return Of::strips(a) || Of::small(a, threads); }
+    static __host__ bool uses_ring(const Args &a)
+    {
+        return (int64_t)a.P * a.H * a.W > 0 && Of::rows16(a) && a.W <= 128 && a.H >= 2;
+    }
     static __device__ void run(const Args &a, const Ctx &cx)
     {
         if ((int64_t)a.P * a.H * a.W == 0) return;
-        const int64_t rows = (int64_t)a.P * ((a.H - 1) / 2 + 1);
-        const bool vec = rows16(a);
-        const bool flat = flat_range((int64_t)a.P * a.H, a.W, cx) &&
-                          !(vec ? per_warp(rows, cx, few_rows(a.W))
-                                : per_thread(rows * ((a.W - 1) / 2 + 1), cx, ring_rows(a) ? 2 : 10));
-        // not flat: also past 2^31 rows, where 16-byte rows keep the strips'
-        // order of maxima, so that a NaN counts alike whatever the size
-        if (vec && (a.W >= kStripCols || !flat)) {
-            if (a.W <= 128 && a.H >= 2 && WarpRing::available(cx, 0) && run_ring(a, cx)) return;
-            run_vec(a, cx);
-        } else if (flat) {
-            if (!flat_ring(a, cx)) flat_global(a, cx);
+        if (Of::rows16(a)) {
+            if (a.W <= 128 && a.H >= 2 && WarpRing::available(cx, 0) && Of::run_ring(a, cx)) return;
+            Of::run_vec(a, cx);
         } else {
-            run_scalar(a, cx);
+            Of::run_scalar(a, cx);
         }
     }
 };
@@ -930,12 +956,24 @@ struct BodyIm2col {
     // there only: beside the flat path they cost pairs capped at 64 registers
     // 100 bytes of spills and 5 to 11 % (histogram + im2col).
     static constexpr int kRingRows = 14;   // rows of a strip item
-    static constexpr int kStripCols = 56;
+    static constexpr int kStripCols = 56, kStripThreads = 32;
     // Up to as many outputs per thread the flat path's start (a dozen
     // divisions and the ring) costs more than a thread per output: 60 rows of
-    // 75 columns, 1 a thread, 3.3 us, flat 5.2; 60 of 337, 5 a thread, 4.3 and
-    // 6.4; 300 of 112, 8 a thread, 5.6 and 3.9.
-    static constexpr int kFewOutputs = 5;
+    // 75 columns, 1 a thread, 3.3 us, flat 5.2; 600 of 30, 4 a thread, 4.1 and
+    // 3.6; 300 of 112, 8 a thread, 5.6 and 3.9.
+    static constexpr int kFewOutputs = 3;
+    static __host__ __device__ bool rows16(const Args &a)
+    {
+        return (a.W & 3) == 0 && a.W <= 64 && aligned16(a.x) && aligned16(a.col);
+    }
+    static __host__ __device__ bool strips(const Args &a, int threads)   // of the interval
+    {
+        return threads <= kStripThreads && rows16(a) && a.W >= kStripCols;
+    }
+    static __host__ __device__ bool small(const Args &a, int64_t threads)   // of the grid
+    {
+        return !rows16(a) && 9 * (int64_t)a.N * a.C * a.H * a.W <= kFewOutputs * threads;
+    }
     static constexpr bool kRingItem = true;
     static constexpr unsigned kRingMinBytes = 4096;   // the stage: one item
     static __host__ bool uses_ring(const Args &a)
@@ -1109,16 +1147,15 @@ struct BodyIm2col {
         return true;
     }
 
-    // One item of the flat path, its pixels from .. n - 1, VEC consecutive ones
-    // per lane.  Shifted
+    // One item of the flat path, VEC consecutive pixels per lane.  Shifted
     // copy k of pixel i lies at k*HW + i of its plane's output, so a warp's
     // stores are contiguous for any W; VEC == 4 (planes of 16-byte
     // multiples, items that start on one) makes them 128-bit and reads
     // three times six values for four pixels -- in one 128-bit and two
     // 32-bit loads where the rows are 16-byte multiples too.
     template <int VEC, class Get>
-    static __device__ __forceinline__ void flat_item(const Args &a, const FlatRows &f, unsigned g0, unsigned from,
-                                                     unsigned n, const Get &get)
+    static __device__ __forceinline__ void flat_item(const Args &a, const FlatRows &f, unsigned g0, unsigned n,
+                                                     const Get &get)
     {
         const int W = (int)f.W;
         const int64_t HW = (int64_t)f.H * W;
@@ -1127,7 +1164,7 @@ struct BodyIm2col {
         float *o0 = a.col + ((int64_t)p0 * 9 * HW + (int64_t)r0 * W);
         if constexpr (VEC == 4)
             if ((W & 3) == 0) {   // the four pixels are of one row
-                for (unsigned i = from + 4 * lane_id(); i < n; i += 128) {
+                for (unsigned i = 4 * lane_id(); i < n; i += 128) {
                     const unsigned lr = f.row_of(i), t = r0 + lr, p = f.plane_of(t);
                     const unsigned c = i - lr * f.W, r = t - p * f.H;
                     const bool le = c == 0, re = c + 4 == f.W;
@@ -1145,7 +1182,7 @@ struct BodyIm2col {
                 }
                 return;
             }
-        for (unsigned i = from + VEC * lane_id(); i < n; i += 32 * VEC) {
+        for (unsigned i = VEC * lane_id(); i < n; i += 32 * VEC) {
             const unsigned lr = f.row_of(i), t = r0 + lr;
             const unsigned p = f.plane_of(t);
             unsigned c = i - lr * f.W, r = t - p * f.H;
@@ -1223,7 +1260,7 @@ struct BodyIm2col {
                 const int64_t g0 = it * f.R, g1 = min(g0 + (int64_t)f.R, rows);
                 const FlatCopy k = copy(it);
                 k.patch(stage, a.x, (g1 + 1) * W + 1, total, r.lane);
-                flat_item<VEC>(a, f, (unsigned)g0, 0, (unsigned)(g1 - g0) * W,
+                flat_item<VEC>(a, f, (unsigned)g0, (unsigned)(g1 - g0) * W,
                                FlatStage{reinterpret_cast<const float *>(stage) + (g0 * W - k.base)});
             });
         r.finish();
@@ -1239,16 +1276,14 @@ struct BodyIm2col {
         const unsigned W = (unsigned)a.W;
         FlatRows f;
         f.init(W, a.H, (unsigned)rows, max(1u, FlatRows::kMaxValues / W), (unsigned)GW, 1);
-        FlatRuns u;
-        u.init(f, GW);
-        for (int64_t it = gw; it < u.items; it += GW) {
-            unsigned from, upto;
-            const unsigned g0 = u.item(f, it, from, upto);
-            flat_item<1>(a, f, g0, from, upto, FlatGlobal{a.x + (int64_t)g0 * W});
+        for (int64_t it = gw; it < f.items(); it += GW) {
+            const int64_t g0 = it * f.R, g1 = min(g0 + (int64_t)f.R, rows);
+            flat_item<1>(a, f, (unsigned)g0, (unsigned)(g1 - g0) * W, FlatGlobal{a.x + g0 * W});
         }
     }
 
-    // One thread per output: few outputs, and tensors of 2^31 rows or more.
+    // One thread per output: few outputs, few long rows, and tensors of 2^31
+    // rows or more.
     static __device__ void run_scalar(const Args &a, const Ctx &cx)
     {
         const int H = a.H, W = a.W;
@@ -1268,27 +1303,49 @@ struct BodyIm2col {
         }
     }
 
-    // STRIPS: with the strip path for a lone warp's interval (N-way schedules)
-    template <bool STRIPS>
+    // SMALL: with the rule on small tensors; NARROW: with strips in intervals of
+    // up to so many threads (a kernel launched alone is chosen by both before
+    // the launch).
+    template <bool SMALL, int NARROW>
     static __device__ __forceinline__ void run_as(const Args &a, const Ctx &cx)
     {
         if ((int64_t)a.N * a.C * a.H * a.W == 0) return;
-        const bool rows16 = (a.W & 3) == 0 && a.W <= 64 && aligned16(a.x) && aligned16(a.col);
         const bool flat = flat_range((int64_t)a.N * a.C * a.H, a.W, cx) &&
-                          (rows16 || !per_thread(9 * (int64_t)a.N * a.C * a.H * a.W, cx, kFewOutputs));
-        if (STRIPS && cx.nthreads == 32 && rows16 && a.W >= kStripCols && WarpRing::available(cx, 0) && run_ring(a, cx))
+                          !(SMALL && small(a, (int64_t)cx.grid * cx.nthreads));
+        if (NARROW && cx.nthreads <= NARROW && strips(a, cx.nthreads) && WarpRing::available(cx, 0) &&
+            run_ring(a, cx))
             return;
         if (flat) {
             const bool v4 = a.W >= 4 && ((int64_t)a.H * a.W & 3) == 0 && aligned16(a.col);
             if (v4 && flat_ring<4>(a, cx)) return;
             if (flat_ring<1>(a, cx)) return;
         }
-        if (rows16) run_vec(a, cx);
-        else if (flat) flat_global(a, cx);
+        if (rows16(a)) run_vec(a, cx);
+        else if (flat && enough_rows((int64_t)a.N * a.C * a.H, cx, 8)) flat_global(a, cx);
         else run_scalar(a, cx);
     }
+};
 
-    static __device__ void run(const Args &a, const Ctx &cx) { run_as<false>(a, cx); }
+// The body without the flat path, as BodyUpsamplePlain.
+struct BodyIm2colPlain {
+    using Of = BodyIm2col;
+    using Args = Of::Args;
+    static constexpr int kId = Of::kId;
+    static __host__ bool pick(const Args &a, int, int64_t threads)
+    {
+        return Of::small(a, threads);
+    }
+    static __host__ bool uses_ring(const Args &a) { return (int64_t)a.N * a.C * a.H * a.W > 0 && Of::rows16(a); }
+    static __device__ void run(const Args &a, const Ctx &cx)
+    {
+        if ((int64_t)a.N * a.C * a.H * a.W == 0) return;
+        if (Of::rows16(a)) {
+            if (WarpRing::available(cx, 0) && Of::run_ring(a, cx)) return;
+            Of::run_vec(a, cx);
+        } else {
+            Of::run_scalar(a, cx);
+        }
+    }
 };
 
 } // namespace hf

@@ -26,6 +26,25 @@
 
 namespace hf {
 
+// Runs body B.  Bodies with more than one path have a run_as<SMALL, NARROW>.
+// SMALL: with the rule on small tensors (a kernel launched alone is chosen by
+// it, and an N-way launch is not small); pairs have it where they may use
+// kWideRegs registers.  NARROW: with the paths of intervals of up to that many
+// threads (im2col's strips).
+constexpr int kWideRegs = 96;
+template <class B, class = void>
+struct RunAs : std::false_type {
+};
+template <class B>
+struct RunAs<B, std::void_t<decltype(&B::template run_as<true, 1>)>> : std::true_type {
+};
+template <class B, bool SMALL, int NARROW>
+__device__ __forceinline__ void run_body(const typename B::Args &a, const Ctx &c)
+{
+    if constexpr (RunAs<B>::value) B::template run_as<SMALL, NARROW>(a, c);
+    else B::run(a, c);
+}
+
 // ------------------------------------------------------------------ single
 template <class B>
 struct SingleParams {
@@ -56,7 +75,7 @@ __device__ __forceinline__ void single_body(const SingleParams<B> &p)
     __syncthreads();
     c.chk_bar = chk_bar;
 #endif
-    B::run(p.a, c);
+    run_body<B, false, 0>(p.a, c);
 }
 
 // A kernel launched alone, with the registers the compiler picks; block
@@ -67,12 +86,10 @@ __global__ void k_single(const __grid_constant__ SingleParams<B> p)
     single_body<B>(p);
 }
 
-// The same with the registers that blocks of T threads leave: for bodies that
-// declare kSingleBlock in place of k_single (the compiler would spend registers
-// that cost larger blocks), for bodies that declare kFullBlock beside it, at
-// 1024 threads, for launches that k_single's registers do not allow.
-template <class B, int T>
-__global__ void __launch_bounds__(T) k_single_block(const __grid_constant__ SingleParams<B> p)
+// The same with the registers that blocks of 1024 threads leave, for bodies
+// that declare kFullBlock: launches that k_single's registers do not allow.
+template <class B>
+__global__ void __launch_bounds__(1024) k_single_full(const __grid_constant__ SingleParams<B> p)
 {
     single_body<B>(p);
 }
@@ -82,24 +99,10 @@ struct FullBlock : std::false_type {
 template <class B>
 struct FullBlock<B, std::void_t<decltype(B::kFullBlock)>> : std::true_type {
 };
-template <class B, class = void>
-struct SingleBlock : std::false_type {
-};
-template <class B>
-struct SingleBlock<B, std::void_t<decltype(B::kSingleBlock)>> : std::true_type {
-};
-template <class B>
-const void *single_func()
-{
-    if constexpr (SingleBlock<B>::value)
-        return reinterpret_cast<const void *>(&k_single_block<B, B::kSingleBlock>);
-    else
-        return reinterpret_cast<const void *>(&k_single<B>);
-}
 template <class B>
 const void *single_full_func()
 {
-    if constexpr (FullBlock<B>::value) return reinterpret_cast<const void *>(&k_single_block<B, 1024>);
+    if constexpr (FullBlock<B>::value) return reinterpret_cast<const void *>(&k_single_full<B>);
     return nullptr;
 }
 
@@ -117,7 +120,7 @@ struct PairParams {
     int ring_stages_low, ring_stages_high;
 };
 
-template <class A, class B>
+template <class A, class B, bool SMALL, int NARROW>
 __device__ __forceinline__ void pair_body(const PairParams<A, B> &p)
 {
     extern __shared__ __align__(128) unsigned char hf_smem[];
@@ -153,21 +156,21 @@ __device__ __forceinline__ void pair_body(const PairParams<A, B> &p)
     c.chk_bar = chk_bar[low ? 0 : 1];
 #endif
     if (low == (p.low_is_a != 0))
-        A::run(p.a, c);
+        run_body<A, SMALL, NARROW>(p.a, c);
     else
-        B::run(p.b, c);
+        run_body<B, SMALL, NARROW>(p.b, c);
 }
 
 template <class A, class B>
 __global__ void k_pair(const __grid_constant__ PairParams<A, B> p)
 {
-    pair_body<A, B>(p);
+    pair_body<A, B, true, 0>(p);
 }
 
 template <class A, class B, int R>
 __global__ void __maxnreg__(R) k_pair_cap(const __grid_constant__ PairParams<A, B> p)
 {
-    pair_body<A, B>(p);
+    pair_body<A, B, (R >= kWideRegs), 0>(p);
 }
 
 // ------------------------------------------------------------------ N-way
@@ -196,19 +199,20 @@ struct NwayParams {
 
 __device__ __forceinline__ unsigned long long global_ns() { return timer_ns(); }
 
+template <int NARROW>
 __device__ __forceinline__ void dispatch(const NwayParams &p, int j, const Ctx &c)
 {
     const unsigned char *args = p.blob + p.args_off[j];
     switch (p.sched_body[j]) {
     case HF_BODY_BN_STATS: BodyBn::run(*reinterpret_cast<const BodyBn::Args *>(args), c); break;
     case HF_BODY_UPSAMPLE2X:
-        BodyUpsample::run(*reinterpret_cast<const BodyUpsample::Args *>(args), c);
+        run_body<BodyUpsample, false, NARROW>(*reinterpret_cast<const BodyUpsample::Args *>(args), c);
         break;
     case HF_BODY_MAXPOOL3S2:
-        BodyMaxpool::run(*reinterpret_cast<const BodyMaxpool::Args *>(args), c);
+        run_body<BodyMaxpool, false, NARROW>(*reinterpret_cast<const BodyMaxpool::Args *>(args), c);
         break;
     case HF_BODY_IM2COL3:
-        BodyIm2col::run_as<true>(*reinterpret_cast<const BodyIm2col::Args *>(args), c);
+        run_body<BodyIm2col, false, NARROW>(*reinterpret_cast<const BodyIm2col::Args *>(args), c);
         break;
     case HF_BODY_HIST256: BodyHist::run(*reinterpret_cast<const BodyHist::Args *>(args), c); break;
     case HF_BODY_PHILOX:
@@ -261,6 +265,7 @@ __device__ __forceinline__ Ctx interval_ctx(const NwayParams &p, int i)
     return c;
 }
 
+template <int NARROW>
 __device__ __forceinline__ void nway_body(const NwayParams &p)
 {
     const int i = p.warp_int[threadIdx.x >> 5];
@@ -270,7 +275,7 @@ __device__ __forceinline__ void nway_body(const NwayParams &p)
         // kernels sharing an interval share its shared slice: the previous
         // one must be done with it before the next starts
         if (j > j0) interval_sync(interval_ctx(p, i));
-        dispatch(p, j, interval_ctx(p, i));
+        dispatch<NARROW>(p, j, interval_ctx(p, i));
     }
     if (p.trace && (threadIdx.x & 31) == 0) atomicMax(p.trace + 2 * i + 1, global_ns());
 }
@@ -279,7 +284,7 @@ __global__ void __launch_bounds__(512) k_nway(const __grid_constant__ NwayParams
 template <int R>
 __global__ void __maxnreg__(R) k_nway_cap(const __grid_constant__ NwayParams p)
 {
-    nway_body(p);
+    nway_body<32>(p);
 }
 
 // ------------------------------------------------------------------ host side
@@ -353,8 +358,11 @@ const Instance *nway_table(int *n);
 // Standalone kernels: one per body, no register bound.
 struct SingleEntry {
     int body;
-    const void *func;        // k_single, or k_single_block
-    const void *func_full;   // k_single_block of 1024 threads, or nullptr
+    const void *func;        // k_single
+    const void *func_full;   // k_single_full, or nullptr
+    const void *plain;       // k_single of the body without its flat path, or nullptr
+    bool (*pick_plain)(const void *args, int block, int64_t threads);   // where that is the one to launch
+    bool (*plain_ring)(const void *args);                               // and whether it uses a ring
     cudaError_t (*launch)(const void *func, const void *args, int threads, int grid, unsigned smem, unsigned *err,
                           unsigned ring_stage, int ring_stages, cudaStream_t);
 };

@@ -538,23 +538,41 @@ void interval_smem_at(const int *ids, const void *const *args, const int *thread
 } // namespace hf
 
 namespace {
-// The kernel of a body launched alone on blocks of `threads`, and its info.
-hf_status single_kernel(const SingleEntry *e, int threads, const void **func, FuncInfo *fi)
+// The kernel that a body is launched alone with on blocks of `threads`, its
+// info and its plan.  A body with a plain kernel has two: which is launched
+// depends on the arguments and the grid that the other one would have.
+hf_status single_kernel(const hf_kernel_t *k, const void *args, int threads, int want, const void **func, FuncInfo *fi,
+                        LaunchPlan *plan)
 {
+    const SingleEntry *e = find_single(k->body);
+    const BodyOps &ops = body_ops(k->body);
+    const size_t base = ops.smem(threads, args);
+    int ring = ops.ring(args);
     *func = e->func;
     hf_status s = func_info(e->func, fi);
-    if (s || fi->max_threads >= threads || !e->func_full) return s;
-    *func = e->func_full;
-    return func_info(e->func_full, fi);
-}
-
-hf_status single_plan(const hf_kernel_t *k, const void *func, const void *args, int threads, int want,
-                      LaunchPlan *plan)
-{
-    const size_t base = body_ops(k->body).smem(threads, args);
-    const int ring = body_ops(k->body).ring(args);
-    const unsigned ring_min = body_ops(k->body).ring_min;
-    return plan_launch(func, threads, 1, &threads, &base, &ring, &ring_min, want, plan);
+    if (s) return s;
+    if (fi->max_threads < threads && e->func_full) {
+        *func = e->func_full;
+        s = func_info(e->func_full, fi);
+        if (s) return s;
+    }
+    FuncInfo pi;
+    if (e->plain) {
+        s = func_info(e->plain, &pi);
+        if (s) return s;
+    }
+    const bool fits = fi->max_threads >= threads, plain_fits = e->plain && pi.max_threads >= threads;
+    if (!fits && !plain_fits)
+        return fail(HF_ERR_REGS, "kernel uses %d registers: at most %d threads", fi->regs, fi->max_threads);
+    if (fits) {
+        s = plan_launch(*func, threads, 1, &threads, &base, &ring, &ops.ring_min, want, plan);
+        if (s) return s;
+        if (!plain_fits || !e->pick_plain(args, threads, (int64_t)plan->grid * threads)) return HF_OK;
+    }
+    *func = e->plain;
+    *fi = pi;
+    ring = e->plain_ring(args) ? kRingItem : kRingNone;
+    return plan_launch(*func, threads, 1, &threads, &base, &ring, &ops.ring_min, want, plan);
 }
 
 hf_status validate_args(int body, const void *a, int which)
@@ -951,12 +969,8 @@ hf_status hf_launch_single(hf_kernel k, const void *args, int threads, int grid,
     const SingleEntry *e = find_single(k->body);
     FuncInfo fi;
     const void *func;
-    s = single_kernel(e, threads, &func, &fi);
-    if (s) return s;
-    if (fi.max_threads < threads)
-        return fail(HF_ERR_REGS, "kernel uses %d registers: at most %d threads", fi.regs, fi.max_threads);
     LaunchPlan plan;
-    s = single_plan(k, func, args, threads, grid, &plan);
+    s = single_kernel(k, args, threads, grid, &func, &fi, &plan);
     if (s) return s;
     HF_CUDA(e->launch(func, args, threads, plan.grid, plan.smem, hf::error_word(), plan.ring_stage[0],
                       plan.ring_stages[0], static_cast<cudaStream_t>(stream)));
@@ -995,13 +1009,10 @@ hf_status hf_query_single(hf_kernel k, const void *args, int threads, hf_fused_i
     if (!k || !args || !info) return fail(HF_ERR_INVALID, "NULL argument");
     hf_status s = check_threads(k, threads);
     if (s) return s;
-    const SingleEntry *e = find_single(k->body);
     FuncInfo fi;
     const void *func;
-    s = single_kernel(e, threads, &func, &fi);
-    if (s) return s;
     LaunchPlan plan;
-    s = single_plan(k, func, args, threads, 0, &plan);
+    s = single_kernel(k, args, threads, 0, &func, &fi, &plan);
     if (s) return s;
     const size_t smem = plan.smem;
     const int bps = plan.bps;

@@ -1,5 +1,5 @@
-"""Tensors of few long rows on the resampling bodies' flat path without a
-ring: rows cut into runs of columns that the warps share."""
+"""Tensors of few rows too long for a ring of the resampling bodies: a thread
+per output below a number of rows per warp, the flat path's items above."""
 import numpy as np
 import pytest
 import torch
@@ -23,9 +23,10 @@ def _out(body, s):
     return torch.full(shape, -7.5, device=DEV)
 
 
-# columns around whole runs (32, 256) and whole shares of a warp
+# long rows, and row counts on both sides of each body's line at these grids
 @pytest.mark.parametrize("shape", [(1, 1, 1, 508), (1, 1, 2, 545), (1, 1, 1, 1015), (1, 2, 3, 1057), (1, 1, 2, 2305),
-                                   (3, 1, 1, 9731), (1, 1, 1, 77825), (1, 1, 5, 15553)])
+                                   (3, 1, 1, 9731), (1, 1, 1, 77825), (1, 1, 5, 15553),
+                                   (2, 61, 5, 509), (1, 153, 2, 1025)])
 @pytest.mark.parametrize("off", [0, 1])
 def test_long_rows(shape, off):
     x, z = W.upsample_input(shape), W.maxpool_input(shape)
@@ -46,8 +47,8 @@ def test_long_rows(shape, off):
 @pytest.mark.parametrize("body", list(ARGS))
 def test_one_row_uses_every_warp(body):
     """The same values as one row and as a thousand rows, neither of which a
-    ring holds, are the same work: the row may not leave warps idle (on one
-    warp it took 100 times as long and more)."""
+    ring holds, are the same work: the row may not be left to one warp (where it
+    took 100 times as long and more)."""
     k = H.hf_register_kernel(body)
     best = []
     for shape in ((1, 1, 1, 1000001), (1, 1, 1000, 1001)):
