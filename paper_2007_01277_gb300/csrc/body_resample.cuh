@@ -948,15 +948,19 @@ struct BodyIm2col {
     static constexpr int kId = HF_BODY_IM2COL3;
     static constexpr int kBarriers = 0;
     // ring path: a stage holds at least three rows (the flat path).  Strips
-    // of whole 16-byte rows, a half-warp a row, take fewer instructions: at W =
-    // 56 and 64 a lone warp an SM took 93 and 89 us for 2^23 values, flat 101
-    // and 108 -- level from two warps on, and strips 1.2 to 4.7 times slower
-    // at W = 48 .. 16.  So they are kept for a lone warp's interval of an
-    // N-way schedule (the 8-way launch 392.9 us, 395.4 without) and compiled
-    // there only: beside the flat path they cost pairs capped at 64 registers
-    // 100 bytes of spills and 5 to 11 % (histogram + im2col).
+    // of whole 16-byte rows, a half-warp a row, take fewer instructions, which
+    // narrow intervals are bound by: 2^22 values with one warp an SM, W = 48 / 56
+    // / 60 / 64, 54 / 41 / 43 / 38 us, flat 51 / 46 / 49 / 50; two warps 29 / 23 /
+    // 26 / 22 and 26 / 26 / 27 / 27; level from three on, and 1.2 to 4.7 times
+    // slower at W = 40 .. 16.  So they take rows of kStripCols columns or more in
+    // intervals of up to kStripThreads.  Beside the flat path they cost kernels
+    // capped at 64 registers 100 bytes of spills and 5 to 11 % (histogram +
+    // im2col; the 8-way launch on eight narrow intervals 552 us, 512 without),
+    // so those are compiled without; and pairs have them in kernels of their own
+    // for blocks with a narrow interval (batch-norm + im2col 64x64, 224 + 32
+    // threads, 14.8 -> 13.1 us), which leaves the other blocks' code alone.
     static constexpr int kRingRows = 14;   // rows of a strip item
-    static constexpr int kStripCols = 56, kStripThreads = 32;
+    static constexpr int kStripCols = 56, kStripThreads = 64;
     // Up to as many outputs per thread the flat path's start (a dozen
     // divisions and the ring) costs more than a thread per output: 60 rows of
     // 75 columns, 1 a thread, 3.3 us, flat 5.2; 600 of 30, 4 a thread, 4.1 and
@@ -1305,7 +1309,8 @@ struct BodyIm2col {
 
     // SMALL: with the rule on small tensors; NARROW: with strips in intervals of
     // up to so many threads (a kernel launched alone is chosen by both before
-    // the launch).
+    // the launch; N-way kernels keep them to one warp: with two the 8-way
+    // launch on eight narrow intervals took 534 us, 528 with one).
     template <bool SMALL, int NARROW>
     static __device__ __forceinline__ void run_as(const Args &a, const Ctx &cx)
     {
@@ -1331,9 +1336,9 @@ struct BodyIm2colPlain {
     using Of = BodyIm2col;
     using Args = Of::Args;
     static constexpr int kId = Of::kId;
-    static __host__ bool pick(const Args &a, int, int64_t threads)
+    static __host__ bool pick(const Args &a, int block, int64_t threads)
     {
-        return Of::small(a, threads);
+        return Of::strips(a, block) || Of::small(a, threads);
     }
     static __host__ bool uses_ring(const Args &a) { return (int64_t)a.N * a.C * a.H * a.W > 0 && Of::rows16(a); }
     static __device__ void run(const Args &a, const Ctx &cx)

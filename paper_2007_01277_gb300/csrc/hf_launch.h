@@ -9,6 +9,7 @@
 namespace hfl {
 
 struct PairLaunch {
+    const void *func;          // the instance's kernel to launch
     const void *const *args;   // [0] body A args, [1] body B args
     int w_split, n_low, n_high;
     unsigned smem_high, smem_total;
@@ -25,6 +26,10 @@ struct Instance {
     int regcap;           // 0 = none
     const void *func;     // the __global__ symbol
     cudaError_t (*launch_pair)(const PairLaunch &, cudaStream_t);
+    // The same with the paths of narrow intervals, for blocks whose interval
+    // of body A (B) has narrow_a (narrow_b) threads or fewer; NULL: none.
+    const void *narrow = nullptr;
+    int narrow_a = 0, narrow_b = 0;
 };
 
 // The pairs compiled with bounded software barriers (inst_checked.cu).

@@ -28,10 +28,11 @@ namespace hf {
 
 // Runs body B.  Bodies with more than one path have a run_as<SMALL, NARROW>.
 // SMALL: with the rule on small tensors (a kernel launched alone is chosen by
-// it, and an N-way launch is not small); pairs have it where they may use
-// kWideRegs registers.  NARROW: with the paths of intervals of up to that many
-// threads (im2col's strips).
-constexpr int kWideRegs = 96;
+// it, and an N-way launch is not small).  NARROW: with the paths of intervals
+// of up to that many threads (im2col's strips).  Pairs and N-way kernels have
+// these where they may use kWideRegs registers; under lower caps each costs
+// the other paths more in spills than it gives.
+constexpr int kWideRegs = 96, kAnyNarrow = 1024;
 template <class B, class = void>
 struct RunAs : std::false_type {
 };
@@ -161,16 +162,16 @@ __device__ __forceinline__ void pair_body(const PairParams<A, B> &p)
         run_body<B, SMALL, NARROW>(p.b, c);
 }
 
-template <class A, class B>
+template <class A, class B, bool NARROW = false>
 __global__ void k_pair(const __grid_constant__ PairParams<A, B> p)
 {
-    pair_body<A, B, true, 0>(p);
+    pair_body<A, B, true, NARROW ? kAnyNarrow : 0>(p);
 }
 
-template <class A, class B, int R>
+template <class A, class B, int R, bool NARROW = false>
 __global__ void __maxnreg__(R) k_pair_cap(const __grid_constant__ PairParams<A, B> p)
 {
-    pair_body<A, B, (R >= kWideRegs), 0>(p);
+    pair_body<A, B, (R >= kWideRegs), NARROW ? kAnyNarrow : 0>(p);
 }
 
 // ------------------------------------------------------------------ N-way
@@ -284,7 +285,7 @@ __global__ void __launch_bounds__(512) k_nway(const __grid_constant__ NwayParams
 template <int R>
 __global__ void __maxnreg__(R) k_nway_cap(const __grid_constant__ NwayParams p)
 {
-    nway_body<32>(p);
+    nway_body<(R >= kWideRegs ? 32 : 0)>(p);
 }
 
 // ------------------------------------------------------------------ host side
@@ -305,7 +306,7 @@ constexpr int compiled_cap(int r)
     return r;
 }
 
-template <class A, class B, int R>
+template <class A, class B, int R, bool NARROW = false>
 const void *pair_func()
 {
 #ifdef HF_CHECKED_BARRIERS
@@ -315,9 +316,9 @@ const void *pair_func()
     else
 #endif
     if constexpr (R == 0)
-        return reinterpret_cast<const void *>(&k_pair<A, B>);
+        return reinterpret_cast<const void *>(&k_pair<A, B, NARROW>);
     else
-        return reinterpret_cast<const void *>(&k_pair_cap<A, B, compiled_cap<A, B>(R)>);
+        return reinterpret_cast<const void *>(&k_pair_cap<A, B, compiled_cap<A, B>(R), NARROW>);
 }
 
 template <class A, class B, int R>
@@ -338,13 +339,31 @@ cudaError_t launch_pair(const PairLaunch &L, cudaStream_t s)
     p.ring_stages_low = L.ring_stages[0];
     p.ring_stages_high = L.ring_stages[1];
     void *kargs[] = {&p};
-    return cudaLaunchKernel(pair_func<A, B, R>(), dim3(L.grid), dim3(L.d0), kargs, L.smem_total, s);
+    return cudaLaunchKernel(L.func, dim3(L.grid), dim3(L.d0), kargs, L.smem_total, s);
 }
+
+// Bodies with paths of their own for narrow intervals declare the interval's
+// threads up to which they are used.
+template <class B, class = void>
+struct NarrowThreads {
+    static constexpr int value = 0;
+};
+template <class B>
+struct NarrowThreads<B, std::void_t<decltype(B::kStripThreads)>> {
+    static constexpr int value = B::kStripThreads;
+};
 
 template <class A, class B, int R>
 Instance make_pair_instance()
 {
-    return Instance{A::kId, B::kId, R, pair_func<A, B, R>(), &launch_pair<A, B, R>};
+    Instance e{A::kId, B::kId, R, pair_func<A, B, R>(), &launch_pair<A, B, R>};
+    constexpr int na = NarrowThreads<A>::value, nb = NarrowThreads<B>::value;
+    if constexpr ((na || nb) && (R == 0 || R >= kWideRegs)) {
+        e.narrow = pair_func<A, B, R, true>();
+        e.narrow_a = na;
+        e.narrow_b = nb;
+    }
+    return e;
 }
 
 // Table accessors implemented by the instantiation units.

@@ -276,6 +276,7 @@ struct hf_fused_t {
     // pair
     int body_low, body_high, n_low, n_high;
     const Instance *inst;
+    const void *func;   // the instance's kernel for this block
     int low_is_a;   // instance body A runs on the low interval
     // N-way
     int n;
@@ -642,7 +643,7 @@ hf_status nway_params(const hf_fused_t *f, const void *const *args, int want, Nw
         }
     }
     p->int_first[f->n_int] = slot;
-    hf_status s = plan_launch(f->inst->func, f->d0, f->n_int, f->int_threads, base, ring, ring_min, want,
+    hf_status s = plan_launch(f->func, f->d0, f->n_int, f->int_threads, base, ring, ring_min, want,
                               plan);
     if (s) return s;
     for (int i = 0; i < f->n_int; ++i) {
@@ -662,7 +663,7 @@ hf_status pair_plan(const hf_fused_t *f, const void *const *uargs, int want, Lau
                             body_ops(f->body_high).smem(f->n_high, uargs[1])};
     const int ring[2] = {body_ops(f->body_low).ring(uargs[0]), body_ops(f->body_high).ring(uargs[1])};
     const unsigned ring_min[2] = {body_ops(f->body_low).ring_min, body_ops(f->body_high).ring_min};
-    return plan_launch(f->inst->func, f->d0, 2, threads, base, ring, ring_min, want, plan);
+    return plan_launch(f->func, f->d0, 2, threads, base, ring, ring_min, want, plan);
 }
 } // namespace
 
@@ -824,8 +825,20 @@ hf_status fuse_pair(hf_kernel a, hf_kernel b, int split, int d0, int regcap, boo
         f->int_threads[0] = split;
         f->int_threads[1] = d0 - split;
     }
+    f->func = f->inst->func;
     FuncInfo fi;
-    s = func_info(f->inst->func, &fi);
+    if (!f->nway && f->inst->narrow) {
+        const int na = f->low_is_a ? f->n_low : f->n_high, nb = f->low_is_a ? f->n_high : f->n_low;
+        if (na <= f->inst->narrow_a || nb <= f->inst->narrow_b) {
+            s = func_info(f->inst->narrow, &fi);
+            if (s) {
+                delete f;
+                return s;
+            }
+            if (fi.max_threads >= d0) f->func = f->inst->narrow;
+        }
+    }
+    s = func_info(f->func, &fi);
     if (s) {
         delete f;
         return s;
@@ -882,6 +895,7 @@ hf_status hf_fuse_n(const hf_kernel *ks, int n, const int *interval_of, const in
     f->regcap = regcap;
     f->d0 = d0;
     f->inst = find_nway(regcap);
+    f->func = f->inst->func;
     f->n = n;
     f->n_int = n_intervals;
     for (int j = 0; j < n; ++j) {
@@ -890,7 +904,7 @@ hf_status hf_fuse_n(const hf_kernel *ks, int n, const int *interval_of, const in
     }
     for (int i = 0; i < n_intervals; ++i) f->int_threads[i] = interval_threads[i];
     FuncInfo fi;
-    hf_status s = func_info(f->inst->func, &fi);
+    hf_status s = func_info(f->func, &fi);
     if (s) {
         delete f;
         return s;
@@ -937,7 +951,7 @@ static hf_status launch_impl(hf_fused f, const void *const *args, int grid, void
         LaunchPlan plan;
         s = pair_plan(f, args, grid, &plan);
         if (s) return s;
-        PairLaunch L{iargs, f->n_low / 32, f->n_low, f->n_high, plan.off[1], plan.smem, f->low_is_a,
+        PairLaunch L{f->func, iargs, f->n_low / 32, f->n_low, f->n_high, plan.off[1], plan.smem, f->low_is_a,
                      plan.grid, f->d0, hf::error_word(), {plan.ring_stage[0], plan.ring_stage[1]},
                      {plan.ring_stages[0], plan.ring_stages[1]}};
         HF_CUDA(f->inst->launch_pair(L, st));
@@ -954,7 +968,7 @@ static hf_status launch_impl(hf_fused f, const void *const *args, int grid, void
     p.trace = trace;
     p.err = hf::error_word();
     void *kargs[] = {&p};
-    HF_CUDA(cudaLaunchKernel(f->inst->func, dim3(plan.grid), dim3(f->d0), kargs, plan.smem, st));
+    HF_CUDA(cudaLaunchKernel(f->func, dim3(plan.grid), dim3(f->d0), kargs, plan.smem, st));
     return HF_OK;
 }
 
@@ -990,7 +1004,7 @@ hf_status hf_query(hf_fused f, const void *const *args, hf_fused_info *info)
         if (s) return s;
     }
     FuncInfo fi;
-    hf_status s = func_info(f->inst->func, &fi);
+    hf_status s = func_info(f->func, &fi);
     if (s) return s;
     const unsigned smem = plan.smem;
     const int bps = plan.bps;
