@@ -233,6 +233,15 @@ __device__ __forceinline__ void put4(unsigned addr, float4 v)
                  : "memory");
 }
 
+// ReLU of samples s .. s + 3; those past the batch are zero, so that the sums
+// over samples add nothing for them, whatever the parameters (an infinite
+// activation times an error of zero would be NaN).
+__device__ __forceinline__ float4 relu4(const float4 &a, int s, int B)
+{
+    return make_float4(s < B ? fmaxf(a.x, 0.f) : 0.f, s + 1 < B ? fmaxf(a.y, 0.f) : 0.f,
+                       s + 2 < B ? fmaxf(a.z, 0.f) : 0.f, s + 3 < B ? fmaxf(a.w, 0.f) : 0.f);
+}
+
 // acc[0..3] += sum over k (ascending) of w[k] * A[k][0..3]; A's rows S apart
 template <int K>
 __device__ __forceinline__ void columns(const float *w, const float *A, float4 &acc)
@@ -372,7 +381,7 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kTrainThreads) k_m
             const float b = T.b1[u];
             float4 a = make_float4(b, b, b, b);
             columns<IN>(T.W1[u], &T.Xt[cur][0][s4], a);
-            a = make_float4(fmaxf(a.x, 0.f), fmaxf(a.y, 0.f), fmaxf(a.z, 0.f), fmaxf(a.w, 0.f));
+            a = relu4(a, s4, B);
 #pragma unroll
             for (int k = 0; k < kCl; ++k) put4(remote(&T.H1[cur][j0 + u][s4], k), a);
         }
@@ -382,7 +391,7 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kTrainThreads) k_m
             const float b = T.b2[u];
             float4 a = make_float4(b, b, b, b);
             columns<HD>(T.W2[u], &T.H1[cur][0][s4], a);
-            a = make_float4(fmaxf(a.x, 0.f), fmaxf(a.y, 0.f), fmaxf(a.z, 0.f), fmaxf(a.w, 0.f));
+            a = relu4(a, s4, B);
 #pragma unroll
             for (int k = 0; k < kCl; ++k) put4(remote(&T.H2[j0 + u][s4], k), a);
         }
