@@ -678,10 +678,17 @@ hf_status hf_mlp_forward(const float *params, const float *X, int n, float *y, v
  * and adam_v are the first and second moment arrays (device, HF_MLP_NPARAMS
  * each, zero for a fresh run); t0 is the number of Adam steps already taken.
  * loss_out[steps] (may be NULL) receives each step's batch loss; grad_out
- * (may be NULL) receives the first step's gradient.  Deterministic. */
+ * (may be NULL) receives the first step's gradient.  Deterministic.  Where the
+ * device, or the partition of it that `stream` belongs to, cannot hold eight
+ * blocks of 94 KB of shared memory in one cluster, one block of 150 KB runs the
+ * steps instead (hf_mlp_train_block: the same results bit for bit, about 4.5
+ * times the time). */
 hf_status hf_mlp_train(float *params, float *adam_m, float *adam_v, const float *X, const float *Y,
                        const int *idx, int steps, int batch, float lr, float beta1, float beta2,
                        float eps, int t0, float *loss_out, float *grad_out, void *stream);
+hf_status hf_mlp_train_block(float *params, float *adam_m, float *adam_v, const float *X, const float *Y,
+                             const int *idx, int steps, int batch, float lr, float beta1, float beta2,
+                             float eps, int t0, float *loss_out, float *grad_out, void *stream);
 int hf_mlp_nparams(void);
 
 /* ------------------------------------------------------------------ */

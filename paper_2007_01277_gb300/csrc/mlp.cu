@@ -10,7 +10,7 @@
 // comment.
 //
 // k_mlp_train runs a whole training run in one launch of one cluster of eight
-// blocks; see its comment.
+// blocks; see its comment.  k_mlp_train_block does it with one block.
 #include <cmath>
 
 #include "kernels.cuh"
@@ -514,6 +514,160 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kTrainThreads) k_m
     }
 }
 
+// The same run on one block, for devices (or partitions of one) that cannot
+// hold the cluster: every parameter and activation in shared memory, a thread
+// per output, rows padded so that lanes that walk samples hit distinct banks.
+// Its sums keep k_mlp_train's order: the same bits, at 37.3 us a step of 64.
+constexpr int kBlockThreads = 512;
+constexpr int SX = IN + 1, SH = HD + 1;   // padded row strides
+struct BlockSmem {
+    float P[NP], M[NP], V[NP], G[NP];
+    float X[kMaxBatch * SX];
+    float H1[kMaxBatch * SH];
+    float H2[kMaxBatch * SH];   // becomes the error at layer 2 after the output's gradient
+    float D1[kMaxBatch * SH];
+    float Y[kMaxBatch], dY[kMaxBatch];
+};
+
+__global__ void __launch_bounds__(kBlockThreads) k_mlp_train_block(
+    float *__restrict__ Pg, float *__restrict__ Mg, float *__restrict__ Vg, const float *__restrict__ X,
+    const float *__restrict__ Y, const int *__restrict__ idx, int steps, int B, float lr, float beta1, float beta2,
+    float eps, int t0, float *__restrict__ loss_out, float *__restrict__ grad_out)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    BlockSmem &S = *reinterpret_cast<BlockSmem *>(smem_raw);
+    const int tid = threadIdx.x, T = kBlockThreads;
+    for (int p = tid; p < NP; p += T) S.P[p] = Pg[p], S.M[p] = Mg[p], S.V[p] = Vg[p];
+    __syncthreads();
+    const float invB = 1.0f / (float)B;
+    const Adam adam{lr, beta1, beta2, eps};
+    for (int step = 0; step < steps; ++step) {
+        const int *rows = idx + (int64_t)step * B;
+        for (int e = tid; e < B * IN; e += T) S.X[e / IN * SX + e % IN] = X[(int64_t)rows[e / IN] * IN + e % IN];
+        for (int s = tid; s < B; s += T) S.Y[s] = Y[rows[s]];
+        __syncthreads();
+        for (int o = tid; o < B * HD; o += T) {
+            const int j = o / B, s = o % B;
+            float a = S.P[OB1 + j];
+            for (int k = 0; k < IN; ++k) a = __fmaf_rn(S.P[OW1 + j * IN + k], S.X[s * SX + k], a);
+            S.H1[s * SH + j] = fmaxf(a, 0.f);
+        }
+        __syncthreads();
+        for (int o = tid; o < B * HD; o += T) {
+            const int j = o / B, s = o % B;
+            float a = S.P[OB2 + j];
+            for (int i = 0; i < HD; ++i) a = __fmaf_rn(S.P[OW2 + j * HD + i], S.H1[s * SH + i], a);
+            S.H2[s * SH + j] = fmaxf(a, 0.f);
+        }
+        __syncthreads();
+        for (int s = tid; s < B; s += T) {
+            float a = S.P[OB3];
+            for (int j = 0; j < HD; ++j) a = __fmaf_rn(S.P[OW3 + j], S.H2[s * SH + j], a);
+            const float e = a - S.Y[s];
+            S.dY[s] = 2.f * e * invB;
+            S.D1[s] = e * e;   // for the loss
+        }
+        __syncthreads();
+        for (int j = tid; j <= HD + 1; j += T) {   // w3's gradient, b3's, and the loss
+            float g = 0.f;
+            if (j < HD)
+                for (int s = 0; s < B; ++s) g = __fmaf_rn(S.dY[s], S.H2[s * SH + j], g);
+            else
+                for (int s = 0; s < B; ++s) g += j == HD ? S.dY[s] : S.D1[s];
+            if (j <= HD) S.G[j < HD ? OW3 + j : OB3] = g;
+            else if (loss_out) loss_out[step] = g * invB;
+        }
+        __syncthreads();
+        for (int o = tid; o < B * HD; o += T) {
+            const int j = o / B, s = o % B;
+            S.H2[s * SH + j] = S.H2[s * SH + j] > 0.f ? S.dY[s] * S.P[OW3 + j] : 0.f;
+        }
+        __syncthreads();
+        for (int o = tid; o < HD * HD; o += T) {
+            float g = 0.f;
+            for (int s = 0; s < B; ++s) g = __fmaf_rn(S.H2[s * SH + o / HD], S.H1[s * SH + o % HD], g);
+            S.G[OW2 + o] = g;
+        }
+        for (int j = tid; j < HD; j += T) {
+            float g = 0.f;
+            for (int s = 0; s < B; ++s) g += S.H2[s * SH + j];
+            S.G[OB2 + j] = g;
+        }
+        for (int o = tid; o < B * HD; o += T) {
+            const int i = o / B, s = o % B;
+            float a = 0.f;
+            for (int j = 0; j < HD; ++j) a = __fmaf_rn(S.H2[s * SH + j], S.P[OW2 + j * HD + i], a);
+            S.D1[s * SH + i] = S.H1[s * SH + i] > 0.f ? a : 0.f;
+        }
+        __syncthreads();
+        for (int o = tid; o < HD * IN; o += T) {
+            float g = 0.f;
+            for (int s = 0; s < B; ++s) g = __fmaf_rn(S.D1[s * SH + o / IN], S.X[s * SX + o % IN], g);
+            S.G[OW1 + o] = g;
+        }
+        for (int j = tid; j < HD; j += T) {
+            float g = 0.f;
+            for (int s = 0; s < B; ++s) g += S.D1[s * SH + j];
+            S.G[OB1 + j] = g;
+        }
+        __syncthreads();
+        const float tf = (float)(t0 + step + 1);
+        const float c[2] = {1.f - powf(beta1, tf), 1.f - powf(beta2, tf)};
+        for (int p = tid; p < NP; p += T) {
+            if (grad_out && step == 0) grad_out[p] = S.G[p];
+            S.P[p] = adam.step(S.P[p], S.M[p], S.V[p], S.G[p], c);
+        }
+        __syncthreads();
+    }
+    for (int p = tid; p < NP; p += T) Pg[p] = S.P[p], Mg[p] = S.M[p], Vg[p] = S.V[p];
+}
+
+// Whether the current device and stream can hold k_mlp_train's cluster.
+bool cluster_fits(size_t smem, cudaStream_t stream)
+{
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = kCl;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(kCl);
+    cfg.blockDim = dim3(kTrainThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, k_mlp_train, &cfg) == cudaSuccess) return n > 0;
+    cudaGetLastError();
+    return false;
+}
+
+hf_status train(bool one_block, float *params, float *adam_m, float *adam_v, const float *X, const float *Y,
+                const int *idx, int steps, int batch, float lr, float beta1, float beta2, float eps, int t0,
+                float *loss_out, float *grad_out, cudaStream_t stream)
+{
+    if (!params || !adam_m || !adam_v || !X || !Y || !idx || steps < 0 || batch < 1 ||
+        batch > kMaxBatch || t0 < 0)
+        return hf::set_last_error(HF_ERR_INVALID, "bad MLP training arguments (batch 1..64)");
+    if (steps == 0) return HF_OK;
+    cudaError_t e = cudaSuccess;
+    if (!one_block) {
+        e = cudaFuncSetAttribute(k_mlp_train, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TrainSmem));
+        if (e == cudaSuccess) one_block = !cluster_fits(sizeof(TrainSmem), stream);
+    }
+    if (one_block && e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_mlp_train_block, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BlockSmem));
+    if (e != cudaSuccess) return hf::set_last_error(HF_ERR_CUDA, cudaGetErrorString(e));
+    if (one_block)
+        k_mlp_train_block<<<1, kBlockThreads, sizeof(BlockSmem), stream>>>(
+            params, adam_m, adam_v, X, Y, idx, steps, batch, lr, beta1, beta2, eps, t0, loss_out, grad_out);
+    else
+        k_mlp_train<<<kCl, kTrainThreads, sizeof(TrainSmem), stream>>>(
+            params, adam_m, adam_v, X, Y, idx, steps, batch, lr, beta1, beta2, eps, t0, loss_out, grad_out);
+    e = cudaGetLastError();
+    return e == cudaSuccess ? HF_OK : hf::set_last_error(HF_ERR_CUDA, cudaGetErrorString(e));
+}
+
 } // namespace
 
 extern "C" {
@@ -536,17 +690,16 @@ hf_status hf_mlp_train(float *params, float *adam_m, float *adam_v, const float 
                        const int *idx, int steps, int batch, float lr, float beta1, float beta2,
                        float eps, int t0, float *loss_out, float *grad_out, void *stream)
 {
-    if (!params || !adam_m || !adam_v || !X || !Y || !idx || steps < 0 || batch < 1 ||
-        batch > kMaxBatch || t0 < 0)
-        return hf::set_last_error(HF_ERR_INVALID, "bad MLP training arguments (batch 1..64)");
-    if (steps == 0) return HF_OK;
-    const size_t smem = sizeof(TrainSmem);
-    cudaError_t e = cudaFuncSetAttribute(k_mlp_train, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return hf::set_last_error(HF_ERR_CUDA, cudaGetErrorString(e));
-    k_mlp_train<<<kCl, kTrainThreads, smem, static_cast<cudaStream_t>(stream)>>>(
-        params, adam_m, adam_v, X, Y, idx, steps, batch, lr, beta1, beta2, eps, t0, loss_out, grad_out);
-    e = cudaGetLastError();
-    return e == cudaSuccess ? HF_OK : hf::set_last_error(HF_ERR_CUDA, cudaGetErrorString(e));
+    return train(false, params, adam_m, adam_v, X, Y, idx, steps, batch, lr, beta1, beta2, eps, t0, loss_out, grad_out,
+                 static_cast<cudaStream_t>(stream));
+}
+
+hf_status hf_mlp_train_block(float *params, float *adam_m, float *adam_v, const float *X, const float *Y,
+                             const int *idx, int steps, int batch, float lr, float beta1, float beta2,
+                             float eps, int t0, float *loss_out, float *grad_out, void *stream)
+{
+    return train(true, params, adam_m, adam_v, X, Y, idx, steps, batch, lr, beta1, beta2, eps, t0, loss_out, grad_out,
+                 static_cast<cudaStream_t>(stream));
 }
 
 int hf_mlp_nparams(void) { return NP; }

@@ -218,6 +218,8 @@ def _load():
         "hf_cost_model_set": (_i32, [_P, _i32, _f32, _f32, ctypes.POINTER(PipePeaks), _i32]),
         "hf_mlp_train": (_i32, [_P, _P, _P, _P, _P, _P, _i32, _i32, _f32, _f32, _f32, _f32, _i32,
                                 _P, _P, _P]),
+        "hf_mlp_train_block": (_i32, [_P, _P, _P, _P, _P, _P, _i32, _i32, _f32, _f32, _f32, _f32, _i32,
+                                      _P, _P, _P]),
         "hf_mlp_nparams": (_i32, []),
         "hf_launch_traced": (_i32, [_P, ctypes.POINTER(_P), _i32, _P, _P]),
         "hf_graph_begin": (_i32, [_P]),
@@ -585,6 +587,13 @@ def hf_mlp_train(params, m, v, X, Y, idx, steps, batch, lr=1e-3, beta1=0.9, beta
     _check("hf_mlp_train", lib.hf_mlp_train(_ptr(params), _ptr(m), _ptr(v), _ptr(X), _ptr(Y),
                                             _ptr(idx), steps, batch, lr, beta1, beta2, eps, t0,
                                             _ptr(loss_out), _ptr(grad_out), _stream_ptr(stream)))
+
+
+def hf_mlp_train_block(params, m, v, X, Y, idx, steps, batch, lr=1e-3, beta1=0.9, beta2=0.999,
+                       eps=1e-8, t0=0, loss_out=None, grad_out=None, stream=None):
+    _check("hf_mlp_train_block", lib.hf_mlp_train_block(_ptr(params), _ptr(m), _ptr(v), _ptr(X), _ptr(Y),
+                                                        _ptr(idx), steps, batch, lr, beta1, beta2, eps, t0,
+                                                        _ptr(loss_out), _ptr(grad_out), _stream_ptr(stream)))
 
 
 def hf_launch_traced(f, args, grid=0, stream=None):
