@@ -238,8 +238,14 @@ __device__ __forceinline__ void put4(unsigned addr, float4 v)
 // activation times an error of zero would be NaN).
 __device__ __forceinline__ float4 relu4(const float4 &a, int s, int B)
 {
-    return make_float4(s < B ? fmaxf(a.x, 0.f) : 0.f, s + 1 < B ? fmaxf(a.y, 0.f) : 0.f,
-                       s + 2 < B ? fmaxf(a.z, 0.f) : 0.f, s + 3 < B ? fmaxf(a.w, 0.f) : 0.f);
+    float4 h = make_float4(fmaxf(a.x, 0.f), fmaxf(a.y, 0.f), fmaxf(a.z, 0.f), fmaxf(a.w, 0.f));
+    if (s + 4 > B) {
+        if (s + 1 > B) h.x = 0.f;
+        if (s + 2 > B) h.y = 0.f;
+        if (s + 3 > B) h.z = 0.f;
+        h.w = 0.f;
+    }
+    return h;
 }
 
 // acc[0..3] += sum over k (ascending) of w[k] * A[k][0..3]; A's rows S apart
