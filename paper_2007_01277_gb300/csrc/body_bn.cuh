@@ -55,6 +55,7 @@ struct BodyBn {
     // ring path: one stage per tile (its <= 3 contiguous runs, HW >= 1024)
     static constexpr bool kRingItem = true;
     static constexpr unsigned kRingMinBytes = kTile * sizeof(float);
+    static __host__ double ring_work(const Args &a) { return 4.0 * a.N * a.C * a.HW; }
     static __host__ bool uses_ring(const Args &a)
     {
         return a.C > 0 && a.N > 0 && a.HW >= 1024 && (a.HW & 3) == 0 && aligned16(a.x);

@@ -218,6 +218,9 @@ struct BodyUpsample {
         if ((int64_t)a.P * a.H * a.W <= 0) return false;
         return strips(a) ? a.W <= 128 : aligned16(a.x) && 3u * a.W + kFlatPad <= kRingMinBytes / 4;
     }
+    // the flat path without one is up to three times slower, strips are not
+    static __host__ bool needs_ring(const Args &a) { return !rows16(a) || a.W < kStripCols; }
+    static __host__ double ring_work(const Args &a) { return 20.0 * a.P * a.H * a.W; }
 
     static __host__ size_t workspace_bytes(const Args &) { return 0; }
     static __host__ size_t smem_bytes(int, const Args &) { return 0; }
@@ -615,6 +618,8 @@ struct BodyMaxpool {
         if ((int64_t)a.P * a.H * a.W <= 0) return false;
         return strips(a) ? a.W <= 128 && a.H >= 2 : ring_rows(a);
     }
+    static __host__ bool needs_ring(const Args &a) { return !strips(a); }   // as in BodyUpsample
+    static __host__ double ring_work(const Args &a) { return 5.0 * a.P * a.H * a.W; }
     // three rows and the rounding fit a stage: what a flat item needs
     static __host__ __device__ bool ring_rows(const Args &a)
     {
@@ -984,6 +989,8 @@ struct BodyIm2col {
     {
         return (int64_t)a.N * a.C * a.H * a.W > 0 && aligned16(a.x) && 3u * a.W + kFlatPad <= kRingMinBytes / 4;
     }
+    static __host__ bool needs_ring(const Args &a) { return !rows16(a); }   // as in BodyUpsample
+    static __host__ double ring_work(const Args &a) { return 40.0 * a.N * a.C * a.H * a.W; }
 
     static __host__ size_t workspace_bytes(const Args &) { return 0; }
     static __host__ size_t smem_bytes(int, const Args &) { return 0; }

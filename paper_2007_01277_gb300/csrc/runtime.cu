@@ -49,6 +49,7 @@ struct BodyOps {
     size_t (*workspace)(const void *);
     int barriers;
     int (*ring)(const void *);    // ring kind for these arguments (RingKind below)
+    double (*ring_work)(const void *);   // item ring: bytes read and written
     unsigned ring_min;            // stream ring: least bytes in flight per warp worth a ring;
                                   // item ring: the stage size (one work item)
     const char *name;
@@ -56,11 +57,15 @@ struct BodyOps {
 
 // How a body uses a bulk-copy ring: not at all; streaming whole tiles of a
 // flat array (any stage size, a share of the SM's bytes in flight); or one
-// work item per stage (a fixed stage of ring_min bytes, two per warp).
-enum RingKind { kRingNone = 0, kRingStream = 1, kRingItem = 2 };
+// work item per stage (a fixed stage of ring_min bytes, two per warp), with
+// register loads of about the same speed in its place or (kRingNeeded) not.
+enum RingKind { kRingNone = 0, kRingStream = 1, kRingItem = 2, kRingNeeded = 3 };
+bool item_ring(int kind) { return kind >= kRingItem; }
 
 // Bodies with a ring path declare `static bool uses_ring(const Args &)`;
-// those that take one work item per stage also declare kRingItem = true.
+// those that take one work item per stage also declare kRingItem = true,
+// `static double ring_work(const Args &)` (bytes read and written) and, where
+// they do much worse without, `static bool needs_ring(const Args &)`.
 template <class B, class = void>
 struct RingItem {
     static constexpr bool value = false;
@@ -70,6 +75,14 @@ struct RingItem<B, std::void_t<decltype(B::kRingItem)>> {
     static constexpr bool value = B::kRingItem;
 };
 template <class B, class = void>
+struct RingNeeded {
+    static bool value(const typename B::Args &) { return false; }
+};
+template <class B>
+struct RingNeeded<B, std::void_t<decltype(B::needs_ring(std::declval<const typename B::Args &>()))>> {
+    static bool value(const typename B::Args &a) { return B::needs_ring(a); }
+};
+template <class B, class = void>
 struct RingTrait {
     static int uses(const void *) { return kRingNone; }
 };
@@ -77,9 +90,18 @@ template <class B>
 struct RingTrait<B, std::void_t<decltype(B::uses_ring(std::declval<const typename B::Args &>()))>> {
     static int uses(const void *p)
     {
-        if (!B::uses_ring(*static_cast<const typename B::Args *>(p))) return kRingNone;
-        return RingItem<B>::value ? kRingItem : kRingStream;
+        const auto &a = *static_cast<const typename B::Args *>(p);
+        if (!B::uses_ring(a)) return kRingNone;
+        return !RingItem<B>::value ? kRingStream : RingNeeded<B>::value(a) ? kRingNeeded : kRingItem;
     }
+};
+template <class B, class = void>
+struct RingWork {
+    static double of(const void *) { return 0.0; }
+};
+template <class B>
+struct RingWork<B, std::void_t<decltype(B::ring_work(std::declval<const typename B::Args &>()))>> {
+    static double of(const void *p) { return B::ring_work(*static_cast<const typename B::Args *>(p)); }
 };
 template <class B, class = void>
 struct RingMin {
@@ -98,7 +120,7 @@ BodyOps ops(const char *name)
                    [](const void *p) { return B::validate(*static_cast<const A *>(p)); },
                    [](int n, const void *p) { return B::smem_bytes(n, *static_cast<const A *>(p)); },
                    [](const void *p) { return B::workspace_bytes(*static_cast<const A *>(p)); },
-                   B::kBarriers, &RingTrait<B>::uses, RingMin<B>::value, name};
+                   B::kBarriers, &RingTrait<B>::uses, &RingWork<B>::of, RingMin<B>::value, name};
 }
 
 const BodyOps &body_ops(int id)
@@ -345,7 +367,7 @@ void ring_choice(int n, const int *warps, const int *kind, const unsigned *ring_
                  const bool *item_ok, bool *use, unsigned *stage, int *stages)
 {
     for (int i = 0; i < n; ++i) {
-        use[i] = b > 0 && (kind[i] == kRingStream || (kind[i] == kRingItem && (!item_ok || item_ok[i])));
+        use[i] = b > 0 && (kind[i] == kRingStream || (item_ring(kind[i]) && (!item_ok || item_ok[i])));
         stage[i] = 0;
         stages[i] = 0;
     }
@@ -364,7 +386,7 @@ void ring_choice(int n, const int *warps, const int *kind, const unsigned *ring_
     ring_geom(F, &sB, &sS);
     for (int i = 0; i < n; ++i) {
         if (!use[i]) continue;
-        if (kind[i] == kRingItem) {
+        if (item_ring(kind[i])) {
             stage[i] = (ring_min[i] + 127u) / 128u * 128u;
             stages[i] = kItemStages;
         } else if (sS > 0) {
@@ -413,26 +435,30 @@ hf_status make_plan(const void *func, int d0, int n, const int *threads, const s
         return fail(HF_ERR_REGS, "block of %d threads with %zu B shared memory cannot be resident", d0,
                     base_total);
     if (want > 0) bmax = std::max(1, std::min(bmax, (want + lim.sm_count - 1) / lim.sm_count));
-    // item intervals, largest ring first: the order in which they give up
-    // their ring when shared memory runs out
+    // Item intervals, largest ring first: the order in which they give up their
+    // rings when shared memory runs out; of a pair the one that needs its ring
+    // (pair_plan) last.
     int drop[HF_MAX_INTERVALS], n_item = 0;
     for (int i = 0; i < n; ++i)
-        if (ring[i] == kRingItem) drop[n_item++] = i;
+        if (item_ring(ring[i])) drop[n_item++] = i;
     std::sort(drop, drop + n_item, [&](int x, int y) {
+        if (n == 2 && ring[x] != ring[y]) return ring[x] == kRingItem;
         return (size_t)threads[x] * ring_min[x] > (size_t)threads[y] * ring_min[y];
     });
+    const bool both = n == 2 && n_item == 2;   // the first, the second, then both
     for (int b = bmax; b >= 0; --b)
-        for (int k = 0; k <= n_item; ++k) {
+        for (int k = 0; k <= n_item + both; ++k) {
             // b == 0: the last resort, no rings at the largest block count.
-            // Item rings that do not fit go, largest first, before the block
-            // count drops; stream intervals whose body wants more in flight
-            // per warp than the SM's share gives drop their ring (register
-            // loads).
+            // Item rings that do not fit go before the block count drops;
+            // stream intervals whose body wants more in flight per warp than
+            // the SM's share gives drop their ring (register loads).
             bool use[HF_MAX_INTERVALS], item_ok[HF_MAX_INTERVALS];
             int warps[HF_MAX_INTERVALS], stages[HF_MAX_INTERVALS];
             unsigned stage[HF_MAX_INTERVALS];
             for (int i = 0; i < n; ++i) warps[i] = threads[i] / 32, item_ok[i] = true;
-            for (int j = 0; j < k; ++j) item_ok[drop[j]] = false;
+            if (both && k == 2) item_ok[drop[1]] = false;
+            else
+                for (int j = 0; j < std::min(k, n_item); ++j) item_ok[drop[j]] = false;
             ring_choice(n, warps, ring, ring_min, b, item_ok, use, stage, stages);
             size_t off = 0;
             for (int i = 0; i < n; ++i) {
@@ -604,15 +630,17 @@ hf_status nway_params(const hf_fused_t *f, const void *const *args, int want, Nw
         // kernels sharing an interval share its ring: item geometry (the
         // largest item) when any of them takes items, a stream share else
         unsigned item_min = 0, stream_min = 0;
+        bool needed = false;
         for (int j = 0; j < f->n; ++j)
             if (f->sched_int[j] == i) {
                 const BodyOps &o = body_ops(f->sched_body[j]);
                 base[i] = std::max(base[i], o.smem(f->int_threads[i], args[j]));
                 const int k = o.ring(args[j]);
-                if (k == kRingItem) item_min = std::max(item_min, o.ring_min);
+                if (item_ring(k)) item_min = std::max(item_min, o.ring_min);
+                if (k == kRingNeeded) needed = true;
                 if (k == kRingStream) stream_min = std::max(stream_min, o.ring_min);
             }
-        if (item_min) ring[i] = kRingItem, ring_min[i] = item_min;
+        if (item_min) ring[i] = needed ? kRingNeeded : kRingItem, ring_min[i] = item_min;
         else if (stream_min) ring[i] = kRingStream, ring_min[i] = stream_min;
     }
     p->warp_begin[f->n_int] = w;
@@ -661,8 +689,19 @@ hf_status pair_plan(const hf_fused_t *f, const void *const *uargs, int want, Lau
     const int threads[2] = {f->n_low, f->n_high};
     const size_t base[2] = {body_ops(f->body_low).smem(f->n_low, uargs[0]),
                             body_ops(f->body_high).smem(f->n_high, uargs[1])};
-    const int ring[2] = {body_ops(f->body_low).ring(uargs[0]), body_ops(f->body_high).ring(uargs[1])};
+    int ring[2] = {body_ops(f->body_low).ring(uargs[0]), body_ops(f->body_high).ring(uargs[1])};
     const unsigned ring_min[2] = {body_ops(f->body_low).ring_min, body_ops(f->body_high).ring_min};
+    // Where a flat path loses by its ring (up to three times), the interval with
+    // fewer bytes a warp gives up its own first (max pool 2851x64x19x6 on 384
+    // threads + im2col 4x96x8x12 on 128, two blocks per SM: 29 us, 49 where max
+    // pool's goes; upsample 931x16x7x7 on 384 + max pool 39x64x9x142 on 128: 12.6
+    // us, 18.7 where max pool's goes).
+    if (item_ring(ring[0]) && item_ring(ring[1]) && (ring[0] == kRingNeeded || ring[1] == kRingNeeded)) {
+        const bool low = body_ops(f->body_low).ring_work(uargs[0]) * threads[1] >=
+                         body_ops(f->body_high).ring_work(uargs[1]) * threads[0];   // the low interval's are more
+        ring[low ? 0 : 1] = kRingNeeded;
+        ring[low ? 1 : 0] = kRingItem;
+    }
     return plan_launch(f->func, f->d0, 2, threads, base, ring, ring_min, want, plan);
 }
 } // namespace
