@@ -533,15 +533,14 @@ struct BodyUpsample {
     static __device__ __forceinline__ void run_as(const Args &a, const Ctx &cx)
     {
         if ((int64_t)a.P * a.H * a.W == 0) return;
-        const bool vec = rows16(a);
-        bool flat = flat_range((int64_t)a.P * a.H, a.W, cx);
-        if (SMALL && small(a, (int64_t)cx.grid * cx.nthreads)) flat = false;
-        if (vec && !(flat && !strips(a))) {
+        const bool flat = flat_range((int64_t)a.P * a.H, a.W, cx) &&
+                          !(SMALL && small(a, (int64_t)cx.grid * cx.nthreads));
+        if (strips(a)) {
             if (a.W <= 128 && WarpRing::available(cx, 0) && run_ring(a, cx)) return;
         } else if (flat && flat_ring(a, cx)) {
             return;
         }
-        if (vec && (a.W >= kStripCols || !flat)) run_vec(a, cx);
+        if (a.W >= kStripCols && rows16(a)) run_vec(a, cx);
         else if (flat && enough_rows((int64_t)a.P * a.H, cx, 12)) flat_global(a, cx);
         else run_scalar(a, cx);
     }
