@@ -31,3 +31,36 @@ def test_same_bits_as_the_cluster(batch):
     for bad in (dict(steps=-1), dict(batch=65), dict(batch=0)):
         with pytest.raises(H.HFError):
             H.hf_mlp_train_block(P, M, V, X, Y, idx, **{"steps": 1, "batch": batch, **bad})
+
+
+def test_captured_run_keeps_the_cluster():
+    """Recorded into a graph the run is the cluster's too: one block would take
+    more than four times as long."""
+    g = torch.Generator().manual_seed(1)
+    X, Y = torch.rand(200, 24, generator=g).to(DEV), torch.rand(200, generator=g).to(DEV)
+    idx = torch.randint(0, 200, (6400,), generator=g, dtype=torch.int32).to(DEV)
+    P = CM.xavier_params(1).to(DEV)
+    M, V = torch.zeros_like(P), torch.zeros_like(P)
+    direct = [t.clone() for t in (P, M, V)]
+    H.hf_mlp_train(*direct, X, Y, idx, 100, 64)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        H.hf_mlp_train(P, M, V, X, Y, idx, 100, 64)
+    graph.replay()
+    torch.cuda.synchronize()
+    for a, b in zip((P, M, V), direct):
+        assert torch.equal(a, b)
+
+    def best(fn):
+        times = []
+        for _ in range(4):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            fn()
+            b.record()
+            b.synchronize()
+            times.append(a.elapsed_time(b))
+        return min(times)
+
+    assert best(graph.replay) < 2 * best(lambda: H.hf_mlp_train(P, M, V, X, Y, idx, 100, 64))
+    assert 2 * best(graph.replay) < best(lambda: H.hf_mlp_train_block(P, M, V, X, Y, idx, 100, 64))
